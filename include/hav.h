@@ -199,11 +199,10 @@ typedef struct {
     int32_t small_points;    /* levels whose every segment has at most this many
                                 points (0..32768; 0: none; default 32768 where
                                 the device launches 8-CTA clusters) run on
-                                thread-block clusters, one cluster of 8 SMs per
-                                segment, the voxel table in distributed shared
-                                memory (same results; one size per pass, settled
-                                steps as in the grid kernel; same conditions as
-                                solo_points) */
+                                thread-block clusters, one cluster of 8 or 16 SMs
+                                per segment, each SM counting another size of the
+                                search (same results; settled steps as in the
+                                grid kernel; same conditions as solo_points) */
     int32_t solo_points;     /* levels whose every segment has at most this many
                                 points (0..4096; 0: none; default 4096) run on
                                 single CTAs, one per segment, its points and
@@ -214,7 +213,7 @@ typedef struct {
                                 the first level within small_points, then on
                                 clusters until the first level within
                                 solo_points that has more segments than the
-                                device runs clusters at once, or at most 1,024
+                                device runs clusters at once, or at most 2,048
                                 points per segment */
     int32_t cluster_ctas;    /* CTAs per cluster of the small_points levels:
                                 0 (default) = 16 where the call's segments all

@@ -137,6 +137,137 @@ __device__ __forceinline__ bool make_grid_axis(float s, float r, float mn, Grid*
     return floor_div(mn, v, &g->fmin[a]);
 }
 
+// floor(RN(x / v)) without a division.  k is an integer within 1 of x / v (the
+// nearest to x * r for any r close to 1 / v), |k| < 2^22; rem = x - k v is then
+// exact: a multiple of ulp(v) / 2 (or x itself, k = 0) of size below 2 v, and
+// fma rounds once.  Away from the integer, |x / v - k| > |k| 2^-23, RN(x / v)
+// lies on the side of k that rem's sign tells.  Near it, RN(x / v) >= k exactly
+// when x / v is at least the midpoint of k and the binary32 number below it
+// (a tie goes to k, whose last bit is 0), k - 2^(e - 24) with e the exponent of
+// that number (k > 0) or of k (k < 0).  Range of v: floor_cells' caller.
+__device__ __forceinline__ float floor_near(float x, float v, float k, float rem) {
+    if (!(fabsf(k) < 4194304.0f) || (k == 0.0f && fabsf(x) <= __fmul_rn(v, 1e-30f) && x != 0.0f))
+        return floorf(__fdiv_rn(x, v));  // (out of range, or a quotient that may underflow)
+    const int kb = __float_as_int(k);
+    const float p = __int_as_float((k > 0.0f ? kb - 1 : kb) & 0x7f800000);  // 2^e (0 for k = 0)
+    const float t = __fmul_rn(v, __fmul_rn(p, 5.9604644775390625e-08f));    // v 2^(e - 24)
+    return rem >= -t ? k : __fsub_rn(k, 1.0f);
+}
+
+// A grid over a level's bounding box [mn, mx], with what the counting loops
+// need to turn a point of the box into its cell's relative indices without
+// divisions or conversions: the cell of every such point lies between the
+// cells of mn and mx (the floor of Eq. 2 is monotone), so with `fast` set
+// (every axis spans fewer than 2^21 cells, 2^-100 < v < 2^100) no point needs a
+// range check.
+struct BoxGrid {
+    Grid g;                    // (r = 0: cell_key divides)
+    float ra[3];               // 1 / v, approximately
+    int ci[3];                 // -(kMagicBits + floor(mn / v)) per axis (floor_bits)
+    float amb;                 // 2^-22 times the largest v: |rem| up to |k| amb (+ amb 2^-70) is near an integer
+    unsigned nx, nxy;          // cells along x, and in an x-y layer (where `cells` is below 2^32)
+    unsigned c0;               // ci[0] + nx ci[1] + nxy ci[2] mod 2^32 (cell_number)
+    int ok, fast;              // the grid is representable; every cell index is in range
+    unsigned long long cells;  // grid cells the box spans
+};
+constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: q + kMagic is kMagic + the integer nearest to q for |q| < 2^22
+constexpr int kMagicBits = 0x4B400000;
+
+// The bits of kMagic + floor(RN(p / v)) per axis for a point of the box of a
+// fast grid; false where an axis is near an integer (one point in 10^4 to 10^5
+// of a scene).  Without conversion or rounding instructions, which run at a
+// fraction of the rate of additions: k = (q + kMagic) - kMagic, and the bits of
+// q + kMagic are kMagicBits + k.  (|q| >= 2^22: |k| amb exceeds v / 2, so the
+// near case takes it.)
+__device__ __forceinline__ bool floor_bits(const float p[3], const float r[3], const float v[3], float amb, int t[3]) {
+    bool ok = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float s = __fadd_rn(__fmul_rn(p[a], r[a]), kMagic);
+        const float k = __fsub_rn(s, kMagic);
+        const float rem = __fmaf_rn(-k, v[a], p[a]);
+        ok = ok && fabsf(rem) > __fmul_rn(__fadd_rn(fabsf(k), 8.4703294725430034e-22f), amb);  // (|k| + 2^-70) amb
+        t[a] = __float_as_int(s) + (__float_as_int(rem) >> 31);
+    }
+    return ok;
+}
+
+// Relative cell indices u = floor(RN(p / v)) - floor(RN(mn / v)) near an integer.
+static __device__ __noinline__ void floor_cells_near(const float p[3], const BoxGrid& B, int u[3]) {
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+        const float k = __fsub_rn(__fadd_rn(__fmul_rn(p[a], B.ra[a]), kMagic), kMagic);
+        const float f = floor_near(p[a], B.g.v[a], k, __fmaf_rn(-k, B.g.v[a], p[a]));
+        u[a] = static_cast<int>(__fsub_rn(f, B.g.fmin[a]));
+    }
+}
+
+__device__ __forceinline__ void floor_cells(const float p[3], const BoxGrid& B, int u[3]) {
+    if (floor_bits(p, B.ra, B.g.v, B.amb, u)) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) u[a] += B.ci[a];
+    } else {
+        floor_cells_near(p, B, u);
+    }
+}
+
+// What a counting loop keeps of a fast grid of fewer than 2^32 - 1 cells in
+// registers, for the number u_x + nx (u_y + ny u_z) of a point's cell.
+constexpr unsigned kNoCell = 0xffffffffu;
+struct CellMap {
+    float r[3], v[3], amb;
+    unsigned nx, nxy, c0;
+    const BoxGrid* b;
+    __device__ __forceinline__ explicit CellMap(const BoxGrid& B)
+        : r{B.ra[0], B.ra[1], B.ra[2]}, v{B.g.v[0], B.g.v[1], B.g.v[2]}, amb(B.amb), nx(B.nx), nxy(B.nxy), c0(B.c0),
+          b(&B) {}
+    // false: near an integer (then near(), below)
+    __device__ __forceinline__ bool fast(const float4& q, unsigned* c) const {
+        const float p[3] = {q.x, q.y, q.z};
+        int t[3];
+        const bool ok = floor_bits(p, r, v, amb, t);
+        *c = c0 + static_cast<unsigned>(t[0]) + nx * static_cast<unsigned>(t[1]) + nxy * static_cast<unsigned>(t[2]);
+        return ok;
+    }
+    __device__ __forceinline__ unsigned near(const float4& q) const {
+        const float p[3] = {q.x, q.y, q.z};
+        int u[3];
+        floor_cells_near(p, *b, u);
+        return static_cast<unsigned>(u[0]) + nx * static_cast<unsigned>(u[1]) + nxy * static_cast<unsigned>(u[2]);
+    }
+};
+
+// One axis of a BoxGrid of size s * r: v, 1 / v, the cell f0 of mn, and the
+// cells the box [mn, mx] has along it (0: 2^21 and more, or not for the loops
+// above).  False: not representable.
+__device__ __forceinline__ bool box_axis(float s, float r, float mn, float mx, float* v_out, float* rv_out, float* f0,
+                                         unsigned* span) {
+    const float v = __fmul_rn(s, r);
+    *v_out = v;
+    *rv_out = 0.0f;
+    *f0 = 0.0f;
+    *span = 0u;
+    if (!(v > 0.0f) || !isfinite(v)) return false;
+    const float rv = __fdividef(1.0f, v);  // (approximate: it only has to find a neighbouring integer)
+    const bool normal = v > 7.8886090522101181e-31f && v < 1.2676506002282294e30f;  // 2^-100, 2^100
+    *rv_out = rv;
+    float f[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const float x = e ? mx : mn;
+        const float k = __fsub_rn(__fadd_rn(__fmul_rn(x, rv), kMagic), kMagic);
+        if (normal && fabsf(k) < 2097152.0f) {
+            f[e] = floor_near(x, v, k, __fmaf_rn(-k, v, x));
+        } else if (!floor_div(x, v, &f[e])) {
+            return e == 1;  // (mx alone: the grid stands, without a span)
+        }
+        if (e == 0) *f0 = f[0];
+    }
+    const float u = __fsub_rn(f[1], f[0]);
+    if (normal && u >= 0.0f && u < 2097152.0f) *span = static_cast<unsigned>(u) + 1u;
+    return true;
+}
+
 // key = u_x | u_y << 21 | u_z << 42 with u = floor(x / v) - floor(min / v).
 __device__ __forceinline__ bool cell_key(const float p[3], const Grid& g, unsigned long long* key,
                                          float f[3]) {

@@ -228,7 +228,11 @@ int small_clusters(int device, int q);
 int launch_small(const Plan& plan, int first_level, int q, int nclusters, cudaStream_t stream);
 // The same on single CTAs (one per segment), for levels of at most kSoloMax points.
 constexpr int kSoloMax = 4096;
-constexpr int kSoloAlone = 1024;  // a single segment this small goes to one CTA, not a cluster
+// A segment this small goes to one CTA, not a cluster, however few there are
+// (measured on GB300, one cloud to a quarter, one CTA / 16-CTA cluster: 1,000
+// points 33-46 / 42-53 us, 1,500 points 37-47 / 44-53, 2,500 points 41-53 /
+// 47-53, 4,096 points 66-79 / 53-62).
+constexpr int kSoloAlone = 2048;
 int launch_solo(const Plan& plan, int first_level, int nblocks, cudaStream_t stream);
 // Grouping around centres (hav_group.cu); the blocks of its cooperative grid build.
 int group_coresident_blocks(int device);
