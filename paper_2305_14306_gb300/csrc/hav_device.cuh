@@ -240,7 +240,7 @@ struct CellMap {
 // One axis of a BoxGrid of size s * r: v, 1 / v, the cell f0 of mn, and the
 // cells the box [mn, mx] has along it (0: 2^21 and more, or not for the loops
 // above).  False: not representable.
-__device__ __forceinline__ bool box_axis(float s, float r, float mn, float mx, float* v_out, float* rv_out, float* f0,
+static __device__ __noinline__ bool box_axis(float s, float r, float mn, float mx, float* v_out, float* rv_out, float* f0,
                                          unsigned* span) {
     const float v = __fmul_rn(s, r);
     *v_out = v;
@@ -453,28 +453,6 @@ __device__ __forceinline__ int smem_insert(unsigned long long* set, unsigned lon
     return -1;
 }
 
-// smem_insert on a set of (1 << log2) slots starting at set (runtime size).
-__device__ __forceinline__ int smem_insert_n(unsigned long long* set, int log2, unsigned long long key, bool* fresh) {
-    const unsigned m = (1u << log2) - 1u;
-    unsigned slot = smem_hash(key, log2);
-    *fresh = false;
-#pragma unroll 1
-    for (int probe = 0; probe < 32; ++probe) {
-        const unsigned long long cur = set[slot];
-        if (cur == key) return static_cast<int>(slot);
-        if (cur == kEmptyKey) {
-            const unsigned long long prev = atomicCAS(set + slot, kEmptyKey, key);
-            if (prev == kEmptyKey) {
-                *fresh = true;
-                return static_cast<int>(slot);
-            }
-            if (prev == key) return static_cast<int>(slot);
-        }
-        slot = (slot + 1) & m;
-    }
-    return -1;
-}
-
 // ------------------------------------------------ Section 3.3 search steps
 // The next size of a search with bracket (lo, hi): a pending first guess,
 // 2 lo while doubling up (the guided start), else the bisection midpoint in
@@ -494,6 +472,7 @@ __device__ __forceinline__ float cand_size(float lo, float hi, bool up, float fi
     const int x = c + 1;
     const int depth = 31 - __clz(x);
     float s = next_size(lo, hi, up, first);
+#pragma unroll 1
     for (int b = depth - 1; b >= 0; --b) {
         if ((x >> b) & 1) {
             lo = s;
@@ -509,12 +488,14 @@ __device__ __forceinline__ float cand_size(float lo, float hi, bool up, float fi
 // Eq. 3 budget of layer l (0-based).
 __device__ __forceinline__ long long layer_budget(long long m, int layers, int ratio, int l) {
     long long S = 0, pw = 1;
+#pragma unroll 1
     for (int i = 0; i < layers; ++i) {
         S += pw;
         pw *= ratio;
     }
     long long used = 0;
     pw = 1;
+#pragma unroll 1
     for (int i = 0; i < layers - 1; ++i) {
         const long long mi = m * pw / S;
         if (i == l) return mi;
@@ -537,10 +518,10 @@ __device__ __forceinline__ T warp_incl_scan(T x) {
 }
 
 // Exclusive scan over the block; *total receives the sum.  All threads call it.
-template <typename T>
+template <typename T, int kBlock = kThreads>
 __device__ T block_excl_scan(T v, T* total, T* scratch /* >= 32 */) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int kWarps = kThreads / 32;
+    constexpr int kWarps = kBlock / 32;
     T x = warp_incl_scan(v);
     if (lane == 31) scratch[wid] = x;
     __syncthreads();

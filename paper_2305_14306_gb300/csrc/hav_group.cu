@@ -23,6 +23,7 @@
 namespace havk {
 namespace {
 
+constexpr int kBuildThreads = 1024;  // of the grid build
 constexpr int kGrpMaxSample = 256;
 constexpr int kScanItems = 4;                        // cells per thread in the scan
 constexpr int kScanBlock = 1024 * kScanItems;       // cells per scan block
@@ -84,7 +85,7 @@ __device__ void setup_grid(GroupGrid* g, float radius, long long budget) {
 // cell counts; a scan of each block's share of the cells; the shares'
 // offsets; the scatter.  Afterwards end[c] holds the end of cell c in list
 // (its start is end[c - 1]).
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kBuildThreads, 1)
     grp_build(const float* pts, long long n, float radius, long long budget, GroupGrid* g, uint32_t* end,
               uint32_t* block_sums, int32_t* list, Barrier* bar, GlobalHdr* gh) {
     __shared__ GroupGrid sg;
@@ -94,8 +95,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ float redf[6][32];
     const int tid = threadIdx.x;
     const unsigned nb = gridDim.x;
-    const long long gtid = blockIdx.x * static_cast<long long>(kThreads) + tid;
-    const long long gstride = static_cast<long long>(nb) * kThreads;
+    const long long gtid = blockIdx.x * static_cast<long long>(kBuildThreads) + tid;
+    const long long gstride = static_cast<long long>(nb) * kBuildThreads;
     if (tid == 0) epoch = 0u;
     for (long long i = gtid; i < budget; i += gstride) end[i] = 0u;
     float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     if (tid < 6) {
         float r = redf[tid][0];
-        for (int w = 1; w < kThreads / 32; ++w) r = (tid < 3) ? fminf(r, redf[tid][w]) : fmaxf(r, redf[tid][w]);
+        for (int w = 1; w < kBuildThreads / 32; ++w) r = (tid < 3) ? fminf(r, redf[tid][w]) : fmaxf(r, redf[tid][w]);
         if (isfinite(r)) atomicMax(&g->box[tid], (tid < 3) ? ~enc_f(r) : enc_f(r));
     }
     if (!grid_sync_impl(bar, gh, nb, &epoch, &flag)) return;
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const long long cb = share * blockIdx.x;
     const long long ce = (cb + share < cells) ? cb + share : cells;
     uint32_t run = 0;
-    for (long long t0 = cb; t0 < ce; t0 += static_cast<long long>(kThreads) * kScanItems) {
+    for (long long t0 = cb; t0 < ce; t0 += static_cast<long long>(kBuildThreads) * kScanItems) {
         uint32_t x[kScanItems], sum = 0;
         for (int k = 0; k < kScanItems; ++k) {
             const long long i = t0 + static_cast<long long>(tid) * kScanItems + k;
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             sum += x[k];
         }
         uint32_t tot;
-        uint32_t before = block_excl_scan<uint32_t>(sum, &tot, scratch);
+        uint32_t before = block_excl_scan<uint32_t, kBuildThreads>(sum, &tot, scratch);
         for (int k = 0; k < kScanItems; ++k) {
             const long long i = t0 + static_cast<long long>(tid) * kScanItems + k;
             if (i < ce) end[i] = run + before;
@@ -164,11 +165,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // the shares before this one, then the offsets
     uint32_t pre = 0;
-    for (unsigned b = tid; b < blockIdx.x; b += kThreads) pre += ld_volatile_u(&block_sums[b]);
+    for (unsigned b = tid; b < blockIdx.x; b += kBuildThreads) pre += ld_volatile_u(&block_sums[b]);
     uint32_t tot;
-    pre = block_excl_scan<uint32_t>(pre, &tot, scratch);  // (only the total matters)
+    pre = block_excl_scan<uint32_t, kBuildThreads>(pre, &tot, scratch);  // (only the total matters)
     const uint32_t off = tot;
-    for (long long i = cb + tid; i < ce; i += kThreads) end[i] += off;
+    for (long long i = cb + tid; i < ce; i += kBuildThreads) end[i] += off;
     if (!grid_sync_impl(bar, gh, nb, &epoch, &flag)) return;
 
     for (long long i = gtid; i < n; i += gstride) {
@@ -418,7 +419,7 @@ __global__ void spacing_grid_query(const float* sub, long long m, const GroupGri
 int group_coresident_blocks(int device) {
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return -1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grp_build, kThreads, 0) != cudaSuccess) return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grp_build, kBuildThreads, 0) != cudaSuccess) return -1;
     if (per_sm < 1) return -1;
     return sms < kMaxBlocks ? sms : kMaxBlocks;  // one block per SM
 }
@@ -442,7 +443,7 @@ int launch_ball_query(const float* points, long long n, const int32_t* centres, 
     GlobalHdr* gh = reinterpret_cast<GlobalHdr*>(ws + lay.ghdr);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(nblocks));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kBuildThreads);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -478,7 +479,7 @@ int launch_spacing_grid(const float* points, long long n, const int32_t* idx, lo
     GlobalHdr* gh = reinterpret_cast<GlobalHdr*>(ws + lay.ghdr);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(nblocks));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kBuildThreads);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -12,7 +12,12 @@
 
 namespace havk {
 
-constexpr int kThreads = 1024;             // threads per block of the persistent kernel (one block per SM)
+// Threads per block of the persistent kernel (one block per SM): with 1,024 a
+// thread has 64 registers, and what does not fit them goes to local memory, for
+// which the 227 KB of shared memory leave hardly any L1.  (Measured on GB300,
+// room of 1,048,576 points, passes of level 0 / 1 / 2: 21.1 / 17.0 / 25.0 us
+// with 1,024 threads, 18.7 / 11.8 / 16.6 us with 512.)
+constexpr int kThreads = 512;
 constexpr int kMaxSegments = 256;          // segments per launch (plan lives in kernel params)
 constexpr int kMaxLevels = 8;
 constexpr int kMaxLayers = 8;

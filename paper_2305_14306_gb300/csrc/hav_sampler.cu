@@ -10,10 +10,12 @@
 //           cell of the bounding box, so that each block's share of the points
 //           is a compact region; later levels inherit the order
 //   layer l = 1..k (Section 3.4, Eq. 3):
-//     pass p   Cnt(P_l, s_p): Eq. 2 voxel keys are first deduplicated in a
-//              block-local shared-memory set, and only keys new to the block
-//              probe the global open-addressed table (atomicCAS); every fresh
-//              global insert is logged so the table can be cleaned slot by slot;
+//     pass p   Cnt(P_l, s_p): a block first finds one point per cell of its own
+//              points in shared memory, without atomics; voxels it holds whole
+//              are counted there, the others meet in global memory, in a bit
+//              per cell of the cloud's box where the table's memory holds
+//              them, else as keys in the open-addressed table; every fresh
+//              insert is logged so the table can be cleaned slot by slot;
 //              the bisection of Section 3.3 is decided identically by every
 //              block from the pass counts (no leader, no host round trip)
 //     select   centre-closest representative per voxel at s*: a block-local
@@ -48,12 +50,22 @@ namespace {
      (static_cast<unsigned>(layer) << 8) | static_cast<unsigned>(pass))
 
 static_assert(kHistBins % kThreads == 0, "the cut-off scan gives each thread whole bins");
-constexpr int kSetSlots = 16384;   // block-local dedupe set of a bisection pass (128 KB + 32 KB list)
-constexpr size_t kPassSmem = static_cast<size_t>(kSetSlots) * 10;
+constexpr int kTilePts = 8192;     // (candidate, point) units of a bisection pass counted together
+constexpr int kPassWords = 54272;  // 16-bit words of its cells, split over the candidates
+constexpr int kAxisTab = 1024;     // entries of the ownership tables of a work item
+constexpr unsigned kMaxOpen = 256; // undecided units that go to the global table as they are
+constexpr int kPassGrids = 16;     // grids of (work item, candidate) prepared together
+// cell numbers, words, two lists, ownership tables
+constexpr size_t kPassSmem = 4 * static_cast<size_t>(kTilePts) + 2 * static_cast<size_t>(kPassWords) +
+                             4 * static_cast<size_t>(kTilePts) + 4 * static_cast<size_t>(kAxisTab);
 constexpr int kSelSlots = 8192;    // block-local argmin table of the selection (128 KB + 16 KB list)
 constexpr size_t kSelSmem = static_cast<size_t>(kSelSlots) * 20;  // + the list of keys that go global
-constexpr size_t kDynSmem = kPassSmem > kSelSmem ? kPassSmem : kSelSmem;
-constexpr int kBucketMin = 1 << 17;
+constexpr size_t kWorkSmem = kPassSmem > kSelSmem ? kPassSmem : kSelSmem;
+// Segments from this size are sorted by Morton cell at level 0: their items then
+// hold most of their voxels whole.  (Measured on GB300, 64 LiDAR clouds of
+// 20,000-200,000 points: 4.42 ms sorted from 2^17, 4.19 from 2^16, 4.06 from
+// 2^14 points; smaller segments run on the small-level kernels by default.)
+constexpr int kBucketMin = 1 << 14;
 // Loads and probes in flight per thread (the kernel's template arguments,
 // one instantiation per pass shape): with 64 registers a thread (one
 // 1024-thread block per SM), deeper batches spill more than they hide
@@ -63,11 +75,30 @@ template <int IF, int PR>
 struct PassShape {
     static constexpr int kInFlight = IF;  // points loaded ahead per thread
     static constexpr int kProbes = PR;    // global first probes issued together per thread
-    static_assert(kSetSlots % (PR * kThreads) == 0 && kSelSlots % (PR * kThreads) == 0,
+    static_assert(kTilePts % (PR * kThreads) == 0 && kSelSlots % (PR * kThreads) == 0,
                   "flush loops take kProbes slots per thread per step");
 };
 
 enum : int { F_ACTIVE = 1, F_SEARCH = 2, F_ACCEPT = 4, F_UP = 8, F_PRE = 16 };
+
+// How a bisection pass counts the distinct cells of a work item at one size:
+// not (no such grid), through one 16-bit word per cell of the item's own box,
+// through hashed words, or key by key in the global table (a key that may be
+// out of range, or 2^32 cells in the item's box).
+enum : int { kCountNone = 0, kCountDirect = 1, kCountHash = 2, kCountKeys = 3 };
+struct ItemGrid {
+    BoxGrid bg;       // over the item's own points' box
+    float seg_fmin[3];
+    int off[3];       // cells from the segment's box to the item's
+    unsigned nslots;  // words
+    int mode;
+    int axis0;        // first entry of its ownership tables (-1: none)
+    // the segment's box: cells along x and in an x-y layer where the table's
+    // memory holds a bit per cell (0: keys)
+    unsigned snx, snxy;
+    int ny, nz;       // cells along y and z of the item's box
+    unsigned mx, mxy; // floor((2^32 - 1) / nx), and / nxy (cell_axes)
+};
 
 struct Smem {
     // level layout
@@ -101,21 +132,21 @@ struct Smem {
     int cprefix[kMaxSegments + 1];
     // per-block logs of fresh global inserts, one per (table set, owned item, candidate)
     int dcnt[kTableSets][kLocalItems][kMaxCand];
-    // candidate grids of a speculative pass, per owned item
-    Grid cgrid[kLocalItems][kMaxCand];
-    int cvalid[kLocalItems][kMaxCand];
+    // grids of a pass, per (owned item, candidate) of a group of items
+    ItemGrid ig[kPassGrids];
+    int leaf[kMaxSegments];         // where the last pass left the subtree: its prepared grids
+    uint32_t ibox[kLocalItems][6];  // box of an owned item's points of this level (~enc(min), enc(max))
     unsigned rbits;
     int ncand;
-    int setc_log2;
     long long tab_stride;
     // scratch
     long long scan_ll[32];
     int scan_i[32];
+    int gcnt[65];
     unsigned scan_u[32];
     float redf[6][32];
     unsigned epoch;
     unsigned list_n;
-    int set_clean;  // 1 when every slot of the block set is empty
     // a bucketed segment (level 0, and for one cloud the levels that keep its
     // order): per work item of the block, the Morton cells [own_lo, own_hi]
     // of the level-0 bucketing (its box own_mn, own_k[a] = 16 / extent) whose
@@ -149,30 +180,44 @@ struct Smem {
     long long m_total;
 };
 
+// The workspace's regions, computed where they are used (the offsets are in the
+// parameter block): held as pointers they cost registers, or local memory
+// where an array of them is indexed at run time.
 struct Dev {
-    Barrier* bar;
-    GlobalHdr* gh;
-    SegHdr* sh;
-    unsigned* clean;
-    LayerState* ls;        // [2][S]
-    uint32_t* hist;        // [2][S][kHistBins]
-    int32_t* psf;          // [S][kMaxBlocks]
-    int32_t* pcmp;         // [kMaxBlocks]
-    int32_t* pitem;        // [kMaxItems]
-    hav_layer_trace* tr;   // [L][S][kMaxLayers]
-    float4* ord[2];        // level input in processing order: x, y, z, level index
-    int32_t* orig[2];      // original (segment-local) index by level index
-    int32_t* posof;        // staged position by level index (current level)
-    uint32_t* taken[2];    // by level index
-    uint32_t* wpre;        // block-local prefix of taken bits per mask word
-    uint32_t* dirty[kTableSets];  // fresh-insert logs, item-owned ranges of the level index space
-    uint32_t* bkt;         // [2][4096] bucket counts, bucket cursors
-    int32_t* prefix;       // [S][kMaxIters] counts at s_hi / 2^(k+1) of this level (-1: none)
-    unsigned long long* tk[kTableSets];
-    unsigned long long* tv;
-    Cand* cand;
-    unsigned long long* ptimes;
-    int ptimes_cap;
+    const Plan& P;
+    template <typename T>
+    __device__ __forceinline__ T* at(size_t offset) const {
+        return reinterpret_cast<T*>(P.ws + offset);
+    }
+    __device__ __forceinline__ Barrier* bar() const { return at<Barrier>(P.lay.barrier); }
+    __device__ __forceinline__ GlobalHdr* gh() const { return at<GlobalHdr>(P.lay.ghdr); }
+    __device__ __forceinline__ SegHdr* sh() const { return at<SegHdr>(P.lay.seghdr); }
+    __device__ __forceinline__ unsigned* clean() const { return at<unsigned>(P.lay.clean); }
+    __device__ __forceinline__ LayerState* ls() const { return at<LayerState>(P.lay.lstate); }  // [2][S]
+    __device__ __forceinline__ uint32_t* hist() const { return at<uint32_t>(P.lay.hist); }      // [2][S][kHistBins]
+    __device__ __forceinline__ int32_t* psf() const { return at<int32_t>(P.lay.partial_sf); }   // [S][kMaxBlocks]
+    __device__ __forceinline__ int32_t* pcmp() const { return at<int32_t>(P.lay.partial_cmp); } // [kMaxBlocks]
+    __device__ __forceinline__ int32_t* pitem() const { return at<int32_t>(P.lay.pitem); }      // [kMaxItems]
+    __device__ __forceinline__ hav_layer_trace* tr() const { return at<hav_layer_trace>(P.lay.trace); }  // [L][S][kMaxLayers]
+    // level input in processing order: x, y, z, level index
+    __device__ __forceinline__ float4* ord(int b) const { return at<float4>(P.lay.ord[b]); }
+    // original (segment-local) index by level index
+    __device__ __forceinline__ int32_t* orig(int b) const { return at<int32_t>(P.lay.orig[b]); }
+    // staged position by level index (current level)
+    __device__ __forceinline__ int32_t* posof() const { return at<int32_t>(P.lay.posof); }
+    __device__ __forceinline__ uint32_t* taken(int b) const { return at<uint32_t>(P.lay.taken[b]); }  // by level index
+    // block-local prefix of taken bits per mask word
+    __device__ __forceinline__ uint32_t* wpre() const { return at<uint32_t>(P.lay.wpre); }
+    // fresh-insert logs, item-owned ranges of the level index space
+    __device__ __forceinline__ uint32_t* dirty(int b) const { return at<uint32_t>(P.lay.dirty[b]); }
+    __device__ __forceinline__ uint32_t* bkt() const { return at<uint32_t>(P.lay.bkt); }  // bucket counts, bucket cursors
+    // [S][kMaxIters] counts at s_hi / 2^(k+1) of this level (-1: none)
+    __device__ __forceinline__ int32_t* prefix() const { return at<int32_t>(P.lay.prefix); }
+    __device__ __forceinline__ unsigned long long* tk(int b) const { return at<unsigned long long>(P.lay.tabk[b]); }
+    __device__ __forceinline__ unsigned long long* tv() const { return at<unsigned long long>(P.lay.tabv); }
+    __device__ __forceinline__ Cand* cand() const { return at<Cand>(P.lay.cand); }
+    __device__ __forceinline__ unsigned long long* ptimes() const { return P.ptimes; }
+    __device__ __forceinline__ int ptimes_cap() const { return P.ptimes_cap; }
 };
 
 // Barrier plus, when phase timing is on, a (time, tag) record from block 0.
@@ -183,42 +228,42 @@ struct Dev {
 // field stays below 2^48 (at most 640 passes per word, each below 2^31).
 constexpr unsigned long long kFusedErr = 1ull << 36;
 
-__device__ __forceinline__ void phase_record(Dev& d, Smem& st, unsigned tag) {
-    if (d.ptimes && blockIdx.x == 0 && threadIdx.x == 0 && st.ntimes < d.ptimes_cap) {
-        d.ptimes[2 * st.ntimes] = globaltimer();
-        d.ptimes[2 * st.ntimes + 1] = tag;
+__device__ __forceinline__ void phase_record(const Dev& d, Smem& st, unsigned tag) {
+    if (d.ptimes() && blockIdx.x == 0 && threadIdx.x == 0 && st.ntimes < d.ptimes_cap()) {
+        d.ptimes()[2 * st.ntimes] = globaltimer();
+        d.ptimes()[2 * st.ntimes + 1] = tag;
         st.ntimes += 1;
     }
 }
 
-__device__ __forceinline__ void fused_arrive(Dev& d, Smem& st, int par, unsigned long long add) {
-    fused_arrive_impl(&d.bar->fused[par], &st.fused_uses[par], add);
+__device__ __forceinline__ void fused_arrive(const Dev& d, Smem& st, int par, unsigned long long add) {
+    fused_arrive_impl(&d.bar()->fused[par], &st.fused_uses[par], add);
 }
 
-__device__ __forceinline__ bool fused_wait(Dev& d, unsigned nblocks, Smem& st, int par, unsigned tag) {
-    const bool ok = fused_wait_impl(&d.bar->fused[par], d.gh, nblocks, &st.fused_uses[par], &st.fused_last[par],
+__device__ __forceinline__ bool fused_wait(const Dev& d, unsigned nblocks, Smem& st, int par, unsigned tag) {
+    const bool ok = fused_wait_impl(&d.bar()->fused[par], d.gh(), nblocks, &st.fused_uses[par], &st.fused_last[par],
                                     &st.fused_delta, &st.flag);
     phase_record(d, st, tag);
     return ok;
 }
 
-__device__ __forceinline__ void grid_arrive(Dev& d, Smem& st) { grid_arrive_impl(d.bar, &st.epoch); }
+__device__ __forceinline__ void grid_arrive(const Dev& d, Smem& st) { grid_arrive_impl(d.bar(), &st.epoch); }
 
-__device__ __forceinline__ bool grid_wait(Dev& d, unsigned nblocks, Smem& st, unsigned tag) {
-    const bool ok = grid_wait_impl(d.bar, d.gh, nblocks, &st.epoch, &st.flag);
+__device__ __forceinline__ bool grid_wait(const Dev& d, unsigned nblocks, Smem& st, unsigned tag) {
+    const bool ok = grid_wait_impl(d.bar(), d.gh(), nblocks, &st.epoch, &st.flag);
     phase_record(d, st, tag);
     return ok;
 }
 
-__device__ __forceinline__ bool grid_sync(Dev& d, unsigned nblocks, Smem& st, unsigned tag) {
-    const bool ok = grid_sync_impl(d.bar, d.gh, nblocks, &st.epoch, &st.flag);
+__device__ __forceinline__ bool grid_sync(const Dev& d, unsigned nblocks, Smem& st, unsigned tag) {
+    const bool ok = grid_sync_impl(d.bar(), d.gh(), nblocks, &st.epoch, &st.flag);
     phase_record(d, st, tag);
     return ok;
 }
 
-__device__ __forceinline__ void seg_error(Dev& d, int s, int code) {
-    atomicCAS(&d.sh[s].status, 0, code);
-    atomicCAS(&d.gh->status, 0, code);
+__device__ __forceinline__ void seg_error(const Dev& d, int s, int code) {
+    atomicCAS(&d.sh()[s].status, 0, code);
+    atomicCAS(&d.gh()->status, 0, code);
 }
 
 // largest s with prefix[s] <= t (prefix has S+1 entries, prefix[0] = 0)
@@ -254,10 +299,10 @@ __device__ __forceinline__ void fill(T* p, long long count, T v, long long gtid,
     for (long long i = gtid; i < count; i += gstride) p[i] = v;
 }
 
-__device__ __forceinline__ void clear_layer_state(Dev& d, int S, int q, long long gtid, long long gstride) {
-    fill<uint32_t>(reinterpret_cast<uint32_t*>(d.ls + q * S), static_cast<long long>(S) * (sizeof(LayerState) / 4),
+__device__ __forceinline__ void clear_layer_state(const Dev& d, int S, int q, long long gtid, long long gstride) {
+    fill<uint32_t>(reinterpret_cast<uint32_t*>(d.ls() + q * S), static_cast<long long>(S) * (sizeof(LayerState) / 4),
                    0u, gtid, gstride);
-    fill<uint32_t>(d.hist + static_cast<long long>(q) * S * kHistBins, static_cast<long long>(S) * kHistBins, 0u,
+    fill<uint32_t>(d.hist() + static_cast<long long>(q) * S * kHistBins, static_cast<long long>(S) * kHistBins, 0u,
                    gtid, gstride);
 }
 
@@ -412,10 +457,7 @@ __device__ void level_setup(const Plan& P, int j, Smem& st) {
         long long chunk = (nl + P.nblocks - 1) / P.nblocks;  // every block gets a share
         if (chunk < P.chunk_min) chunk = P.chunk_min;
         const int ncand = (1 << depth) - 1;
-        int lg2 = 0;
-        while ((1 << (lg2 + 1)) * ncand <= kSetSlots) ++lg2;
-        // a candidate's share of the block set must stay at most half full
-        const long long half = (1ll << lg2) / 2;
+        const long long half = kTilePts / (depth > 1 ? ncand : 1);  // the units of an item make one tile
         if (depth > 1 && chunk > half) chunk = half;
         long long items = (s < S) ? (n + chunk - 1) / chunk : 0;
         if (depth == 1 && chunk > half) {
@@ -441,12 +483,596 @@ __device__ void level_setup(const Plan& P, int j, Smem& st) {
                 st.chunk = static_cast<int>(chunk);
                 st.tab_stride = stride;
                 st.ncand = ncand;
-                st.setc_log2 = lg2;
             }
             break;
         }
     }
     __syncthreads();
+}
+
+constexpr size_t kDynSmem = kWorkSmem + sizeof(Smem);
+static_assert(kDynSmem <= 227 * 1024, "shared memory of one block");
+static_assert(kWorkSmem % 16 == 0, "alignment of the state behind the work area");
+
+extern __shared__ __align__(16) unsigned char dyn[];
+__device__ __forceinline__ Smem& smem_state() { return *reinterpret_cast<Smem*>(dyn + kWorkSmem); }
+
+// Bits 0, 3, 6, 9 of a bucket coordinate's Morton code.
+__device__ __forceinline__ unsigned dilate4(unsigned c) {
+    return (c & 1u) | ((c & 2u) << 2) | ((c & 4u) << 4) | ((c & 8u) << 6);
+}
+
+// The Morton cells, along axis a, that the points of cell f of a grid of size v
+// can fall in (voxel_owned): the dilated codes of the first and the last one.
+__device__ __forceinline__ unsigned axis_cells(float f, float v, float mn, float k, int a) {
+    float lo = __fmul_rn(v, f);
+    float hi = __fmul_rn(v, __fadd_rn(f, 1.0f));
+    lo = __fsub_rn(lo, __fmul_rn(__fadd_rn(fabsf(lo), v), 9.5367431640625e-07f));
+    hi = __fadd_rn(hi, __fmul_rn(__fadd_rn(fabsf(hi), v), 9.5367431640625e-07f));
+    float tl = __fsub_rn(__fmul_rn(__fsub_rn(lo, mn), k), 0.01f);
+    float th = __fadd_rn(__fmul_rn(__fsub_rn(hi, mn), k), 0.01f);
+    tl = fminf(fmaxf(tl, 0.0f), 15.0f);  // NaN-free: finite inputs
+    th = fminf(fmaxf(th, 0.0f), 15.0f);
+    return (dilate4(static_cast<unsigned>(tl)) << a) | (dilate4(static_cast<unsigned>(th)) << (16 + a));
+}
+
+// f(i, p) for the input points [a, b) of the call, p the coordinates; four
+// points' loads in flight per thread.
+template <typename F>
+__device__ __forceinline__ void for_points(const float* points, int a, int b, F&& f) {
+#pragma unroll 1
+    for (int i0 = a + static_cast<int>(threadIdx.x); i0 < b; i0 += 4 * kThreads) {
+        float p[4][3];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float* q = points + 3 * min(i0 + k * kThreads, b - 1);
+#pragma unroll
+            for (int a3 = 0; a3 < 3; ++a3) p[k][a3] = __ldg(q + a3);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i0 + k * kThreads < b) f(i0 + k * kThreads, p[k]);
+    }
+}
+
+// The boxes of this block's work items of the level, from their points.
+__device__ __noinline__ void item_boxes(int S, unsigned nb, const float4* ord) {
+    Smem& st = smem_state();
+    const int tid = threadIdx.x;
+    if (tid < kLocalItems * 6) (&st.ibox[0][0])[tid] = 0u;
+    __syncthreads();
+    int li = 0;
+    for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
+        int a, b;
+        item_range(st, S, it, &a, &b);
+        float mnv[3] = {INFINITY, INFINITY, INFINITY}, mxv[3] = {-INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 4
+        for (int i = a + tid; i < b; i += kThreads) {
+            const float4 q = ord[i];
+            const float p[3] = {q.x, q.y, q.z};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                mnv[k] = fminf(mnv[k], p[k]);
+                mxv[k] = fmaxf(mxv[k], p[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {  // (a segment with a coordinate that is not finite is not searched)
+            const uint32_t lo = __reduce_max_sync(0xffffffffu, isfinite(mnv[k]) ? ~enc_f(mnv[k]) : 0u);
+            const uint32_t hi = __reduce_max_sync(0xffffffffu, isfinite(mxv[k]) ? enc_f(mxv[k]) : 0u);
+            if ((tid & 31) == 0) {
+                if (lo) atomicMax(&st.ibox[li][k], lo);
+                if (hi) atomicMax(&st.ibox[li][3 + k], hi);
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// The state of a search at leaf l of its subtree (the l-th of the ncand + 1
+// outcomes of a pass; the steps are cand_size's).
+__device__ __forceinline__ void leaf_state(float* lo, float* hi, bool* up, float first, int leaf, int ncand) {
+    const int x = ncand + 1 + leaf;
+    const int depth = 31 - __clz(x);
+    float s = next_size(*lo, *hi, *up, first);
+#pragma unroll 1
+    for (int b = depth - 1; b >= 0; --b) {
+        if ((x >> b) & 1) {
+            *lo = s;
+        } else {
+            *hi = s;
+            *up = false;
+        }
+        s = next_size(*lo, *hi, *up, 0.0f);
+    }
+}
+
+// Grids of (work item, candidate) pairs into st.ig: three lanes (one per axis)
+// a pair, ten pairs a warp, by the warps from w0 on.  leaves = 0: of the items
+// from the block's item li0 on, at the search's state; else of all the block's
+// items at every one of the `leaves` states that the running pass may lead to
+// (pairs item-major, then leaf, then candidate).
+__device__ __noinline__ void item_grids(int S, unsigned nb, int w0, int li0, int count, int leaves, float r0, float r1,
+                                        float r2) {
+    Smem& st = smem_state();
+    const int lane = threadIdx.x & 31;
+    const int wid = static_cast<int>(threadIdx.x >> 5) - w0;
+    if (wid < 0 || wid * 10 >= count) return;  // (warp-uniform)
+    const int o = lane < 30 ? lane / 3 : 9, ax = lane < 30 ? lane - 3 * o : 0, lead = 3 * o;
+    const int ncand = st.ncand;
+    const int e = wid * 10 + o;
+    const int ee = e < count ? e : count - 1;
+    const int c = ee % ncand;
+    const int lf = leaves ? ee / ncand % leaves : 0;
+    const int li = leaves ? ee / (ncand * leaves) : li0 + ee / ncand;
+    const int it = static_cast<int>(blockIdx.x + static_cast<unsigned>(li) * nb);
+    const int s = S == 1 ? 0 : find_seg(st.item0, S, it);
+    const bool search = (st.flags[s] & F_SEARCH) != 0;
+    float lo = st.lo[s], hi = st.hi[s], first = st.first[s];
+    bool up = (st.flags[s] & F_UP) != 0;
+    if (leaves) {
+        leaf_state(&lo, &hi, &up, first, lf, ncand);
+        first = 0.0f;
+    }
+    const float sc = cand_size(lo, hi, up, first, c);
+    const float r = ax == 0 ? r0 : (ax == 1 ? r1 : r2);
+    float v, rv, f0, fs;
+    unsigned span, sspan;
+    const bool ok = box_axis(sc, r, st.mn[s][ax], st.mx[s][ax], &v, &rv, &fs, &sspan);
+    box_axis(sc, r, dec_f(~st.ibox[li][ax]), dec_f(st.ibox[li][3 + ax]), &v, &rv, &f0, &span);
+    const unsigned okm = __ballot_sync(0xffffffffu, ok) >> lead;
+    const unsigned fm = __ballot_sync(0xffffffffu, sspan != 0u && span != 0u) >> lead;
+    const unsigned nx = __shfl_sync(0xffffffffu, span, lead), ny = __shfl_sync(0xffffffffu, span, lead + 1),
+                   nz = __shfl_sync(0xffffffffu, span, lead + 2);
+    const unsigned sx = __shfl_sync(0xffffffffu, sspan, lead), sy = __shfl_sync(0xffffffffu, sspan, lead + 1),
+                   sz = __shfl_sync(0xffffffffu, sspan, lead + 2);
+    const int ci = (fabsf(f0) < 4194304.0f) ? -(kMagicBits + static_cast<int>(f0)) : 0;
+    const unsigned part = static_cast<unsigned>(ci) * (ax == 0 ? 1u : (ax == 1 ? nx : nx * ny));
+    const unsigned c0 = part + __shfl_sync(0xffffffffu, part, lead + 1) + __shfl_sync(0xffffffffu, part, lead + 2);
+    const float vmax = fmaxf(v, fmaxf(__shfl_sync(0xffffffffu, v, lead + 1), __shfl_sync(0xffffffffu, v, lead + 2)));
+    if (e >= count || lane >= 30) return;
+    ItemGrid& g = st.ig[e];
+    g.bg.g.v[ax] = v;
+    g.bg.g.r[ax] = 0.0f;
+    g.bg.g.fmin[ax] = f0;
+    g.bg.ra[ax] = rv;
+    g.bg.ci[ax] = ci;
+    g.seg_fmin[ax] = fs;
+    g.off[ax] = static_cast<int>(__fsub_rn(f0, fs));
+    if (ax == 0) {
+        const bool all_ok = search && (okm & 7u) == 7u, fast = all_ok && (fm & 7u) == 7u;
+        const unsigned long long cells = static_cast<unsigned long long>(nx) * ny * nz;
+        const unsigned long long scells = static_cast<unsigned long long>(sx) * sy * sz;
+        const unsigned words = static_cast<unsigned>(kPassWords / ncand);
+        g.bg.amb = __fmul_rn(vmax, 2.384185791015625e-07f);  // 2^-22
+        g.bg.nx = nx;
+        g.bg.nxy = nx * ny;
+        g.bg.c0 = c0;
+        g.bg.cells = cells;
+        g.ny = static_cast<int>(ny);
+        g.nz = static_cast<int>(nz);
+        g.mx = nx ? 0xffffffffu / nx : 0u;
+        g.mxy = nx * ny ? 0xffffffffu / (nx * ny) : 0u;
+        g.nslots = cells <= words ? static_cast<unsigned>(cells) : words;
+        g.mode = !all_ok ? kCountNone
+                         : (!fast || cells >= kNoCell ? kCountKeys : (cells <= words ? kCountDirect : kCountHash));
+        const bool bits = scells < kNoCell && scells <= (64ull << st.cap_log2[s]);
+        g.snx = bits ? sx : 0u;
+        g.snxy = sx * sy;
+        // (two candidates and more share the tables' room)
+        const unsigned long long ends = static_cast<unsigned long long>(nx) + ny + nz;
+        g.axis0 = (fast && st.own_on[li] && ends <= static_cast<unsigned>(kAxisTab / ncand)) ? (kAxisTab / ncand) * c : -1;
+    }
+}
+
+// c / d and c % d with m = floor((2^32 - 1) / d): the high product is at most two short.
+__device__ __forceinline__ unsigned div_mod(unsigned c, unsigned d, unsigned m, unsigned* rem) {
+    unsigned q = __umulhi(c, m);
+    unsigned r = c - q * d;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (r >= d) {
+            r -= d;
+            ++q;
+        }
+    *rem = r;
+    return q;
+}
+
+// The cell's indices along the axes.
+__device__ __forceinline__ void cell_axes(unsigned c, const ItemGrid& g, unsigned u[3]) {
+    unsigned rest;
+    u[2] = div_mod(c, g.bg.nxy, g.mxy, &rest);
+    u[1] = div_mod(rest, g.bg.nx, g.mx, &u[0]);
+}
+
+// The units of a tile whose cells or keys leave the ranges of pass_items, key
+// by key into the global tables (a function of its own: seldom used).
+__device__ __noinline__ int pass_keys(const float4* ord, const ItemGrid* ig, int ncand, int a, int ia, int L, int li,
+                                      int s, int X, unsigned long long* tk, uint32_t* dirty, long long dstride) {
+    Smem& st = smem_state();
+    const int tid = threadIdx.x, lane = tid & 31;
+    const long long tstride = st.tab_stride;
+    unsigned rbits = 0;  // candidates with a key out of range
+    int bad = 0;
+#pragma unroll 1
+    for (int w0 = tid - lane; w0 < L * ncand; w0 += kThreads) {  // warp-uniform
+        const int w = w0 + lane;
+        const int c = w < L * ncand ? w / L : 0;
+        bool in = w < L * ncand && ig[c].mode != kCountNone;
+        unsigned long long key = 0;
+        if (in) {
+            const float4 q = ord[a + w - c * L];
+            in = __float_as_int(q.w) >= 0;
+            if (in) {
+                const float p[3] = {q.x, q.y, q.z};
+                float f[3];
+                Grid g = ig[c].bg.g;
+                for (int k = 0; k < 3; ++k) g.fmin[k] = ig[c].seg_fmin[k];  // the segment's grid
+                if (!cell_key(p, g, &key, f)) {
+                    rbits |= 1u << c;
+                    in = false;
+                }
+            }
+        }
+        bool fr = false;
+        long long slot = -1;
+        if (in) {
+            slot = find_or_insert(tk + st.tab_off[s] + c * tstride, st.cap_log2[s], key, &fr);
+            if (slot < 0) bad = HAV_ERR_TABLE_FULL;
+        }
+        const bool fresh = in && slot >= 0 && fr;
+        const int k = warp_append_keyed(fresh, c, st.dcnt[X][li]);
+        if (fresh) dirty[c * dstride + ia + k] = static_cast<uint32_t>(c * tstride + st.tab_off[s] + slot);
+    }
+    if (rbits) atomicOr(&st.rbits, rbits);
+    return bad;
+}
+// find_or_insert with a compare-and-swap for every probe (one round trip where
+// the first slot is empty or holds the key); bit 62 of the result: fresh.
+__device__ __noinline__ long long insert_key(unsigned long long* T, int cap_log2, unsigned long long key) {
+    const unsigned mask = (1u << cap_log2) - 1u;
+    unsigned slot = static_cast<unsigned>(slot_mix(key) >> (64 - cap_log2));
+#pragma unroll 1
+    for (unsigned probe = 0; probe <= mask; ++probe) {
+        const unsigned long long cur = atomicCAS(T + slot, kEmptyKey, key);
+        if (cur == kEmptyKey) return static_cast<long long>(slot) | (1ll << 62);
+        if (cur == key) return static_cast<long long>(slot);
+        slot = (slot + 1) & mask;
+    }
+    return -1;
+}
+
+// A bisection pass over this block's work items: Cnt(P_l, s_c) for every
+// candidate c.  Per tile of an item, (a) every point writes its cell number and
+// its unit's index into its cell's word, and the unit that reads its own index
+// back stands for the cell (hashed words: where another cell's index is read
+// back, the unit is undecided); (b)
+// those units are listed; a voxel that the item holds whole is counted here;
+// (c) the others' keys go to the candidates' global tables, kProbes
+// compare-and-swaps in flight per thread.  A function of its own, so that its
+// loops have the whole register budget.
+//
+// Against 64-bit keys inserted with compare-and-swap into a block-local table,
+// the point loop takes a quarter of the instructions (no 64-bit arithmetic, no
+// range checks, no division, no probing), the ownership test one table look-up
+// per axis instead of its arithmetic per key, and the global tables one round
+// trip where a bit stands for a cell.  The next pass's grids are ready before a
+// pass starts (item_grids).  A pass is bound by latency: of a level-0 pass of
+// the 1M-point room (17 us, 21.5 us before), 2.6 us are the points, 2.2 the
+// list, 1.6 the ownership, 2.5 the global tables, 4 the barrier with the wait
+// for the slowest block, the rest short sections between block barriers.
+// Measured on GB300, whole calls: room of 1M points, four levels 836 -> 770 us,
+// room of 300,007 points, guided 479 -> 422 us, 64 LiDAR clouds, two levels
+// 4.36 -> 3.55 ms, ten served scenes 1.03 -> 0.87 ms.
+template <int kProbes, bool kOne>
+__device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, unsigned long long* tk, uint32_t* dirty,
+                                        int X, long long dstride, LayerState* ls, int cslot, SegHdr* sh, GlobalHdr* gh,
+                                        bool prepared, float r0, float r1, float r2) {
+    constexpr int kIn = 4;
+    constexpr int kPer = kTilePts / kThreads;  // units of a tile per thread
+    static_assert(kPer % kIn == 0 && kPer <= 32, "one bit per unit");
+    Smem& st = smem_state();
+    uint32_t* const cell = reinterpret_cast<uint32_t*>(dyn);
+    unsigned short* const word = reinterpret_cast<unsigned short*>(cell + kTilePts);
+    unsigned short* const list = word + kPassWords;
+    unsigned short* const rest = list + kTilePts;
+    uint32_t* const axis = reinterpret_cast<uint32_t*>(rest + kTilePts);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int ncand = kOne ? 1 : st.ncand;
+    const long long tstride = st.tab_stride;
+    const unsigned words = static_cast<unsigned>(kPassWords / ncand);
+    const int group = kPassGrids / ncand;  // items prepared together
+    int li = 0;
+    for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
+        if (!prepared && li % group == 0) {
+            const int left = (st.items_total - it + static_cast<int>(nb) - 1) / static_cast<int>(nb);
+            __syncthreads();  // (every thread is done with the previous group)
+            item_grids(S, nb, 0, li, (left < group ? left : group) * ncand, 0, r0, r1, r2);
+            __syncthreads();
+        }
+        int ia, ib;
+        const int s = item_range(st, S, it, &ia, &ib);
+        if (!(st.flags[s] & F_SEARCH)) continue;
+        const ItemGrid* const ig =
+            st.ig + (prepared ? li * (ncand + 1) + st.leaf[s] : li % group) * ncand;
+        const int cap = st.cap_log2[s];
+        unsigned long long* const Tb = tk + st.tab_off[s];
+        if (tid == 0) st.rbits = 0u;
+        if (tid < kMaxCand) st.xcnt[tid] = 0u;
+        int bad = 0;
+        // a fresh insert's slot into the item's log of its candidate (whole warp calls)
+        auto log_fresh = [&](bool fresh, int c, long long slot) {
+            const int k = kOne ? warp_append(fresh, &st.dcnt[X][li][0]) : warp_append_keyed(fresh, c, st.dcnt[X][li]);
+            if (fresh) dirty[c * dstride + ia + k] = static_cast<uint32_t>(c * tstride + st.tab_off[s] + slot);
+        };
+        bool keys = false, none = true, hashed = false;  // (uniform)
+        for (int c = 0; c < ncand; ++c) {
+            keys = keys || ig[c].mode == kCountKeys;
+            hashed = hashed || ig[c].mode == kCountHash;
+            none = none && ig[c].mode == kCountNone;
+        }
+        const int tile = kTilePts / ncand;
+        // the ownership tables of the item's grids (one tile only: a voxel counted
+        // here is not seen again)
+        const bool own = ib - ia <= tile && !keys && st.own_on[li] != 0;
+        if (own)
+            for (int c = 0; c < ncand; ++c) {
+                const ItemGrid& g = ig[c];
+                if (g.axis0 < 0 || g.mode == kCountNone) continue;
+                const int nx = static_cast<int>(g.bg.nx), ny = g.ny, nz = g.nz;
+#pragma unroll 1
+                for (int k = tid; k < nx + ny + nz; k += kThreads) {
+                    const int a = k < nx ? 0 : (k < nx + ny ? 1 : 2);
+                    const int u = k - (a > 0 ? nx : 0) - (a > 1 ? ny : 0);
+                    axis[g.axis0 + k] = axis_cells(__fadd_rn(g.bg.g.fmin[a], static_cast<float>(u)), g.bg.g.v[a],
+                                                   st.own_mn[li][a], st.own_k[li][a], a);
+                }
+            }
+        for (int a = ia; a < ib && !none; a += tile) {
+            const int L = (ib - a < tile) ? ib - a : tile;
+            const int units = L * ncand;
+            if (tid == 0) {
+                st.list_n = 0u;
+                st.rest_n = 0u;
+            }
+            if (keys) {
+                __syncthreads();
+                bad |= pass_keys(ord, ig, ncand, a, ia, L, li, s, X, tk, dirty, dstride);
+                __syncthreads();
+                continue;
+            }
+            // (a) cells and indices
+            unsigned mult = 0x9E3779B1u;
+            {
+                CellMap map(ig[0].bg);
+                int c1 = 0;
+#pragma unroll 1
+                for (int w0 = tid; w0 < units; w0 += kIn * kThreads) {
+                    float4 q[kIn];
+                    unsigned cn[kIn];
+                    int cc[kIn];
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        const int w = min(w0 + k * kThreads, units - 1);
+                        cc[k] = kOne ? 0 : w / L;
+                        q[k] = ord[a + w - cc[k] * L];
+                    }
+                    unsigned near = 0u;  // points near a cell's face: one branch for all of them
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        if (!kOne && cc[k] != c1) {
+                            c1 = cc[k];
+                            map = CellMap(ig[c1].bg);
+                        }
+                        near |= map.fast(q[k], &cn[k]) ? 0u : (1u << k);
+                    }
+                    if (near) {
+#pragma unroll
+                        for (int k = 0; k < kIn; ++k)
+                            if ((near >> k) & 1u) cn[k] = CellMap(ig[cc[k]].bg).near(q[k]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        const int w = w0 + k * kThreads;
+                        const ItemGrid& g = ig[cc[k]];
+                        if (__float_as_int(q[k].w) < 0 || (!kOne && g.mode == kCountNone)) cn[k] = kNoCell;  // taken
+                        if (w < units) {
+                            cell[w] = cn[k];
+                            if (cn[k] != kNoCell)
+                                word[cc[k] * words + (g.mode == kCountHash ? __umulhi(cn[k] * mult, g.nslots) : cn[k])] =
+                                    static_cast<unsigned short>(w);
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+            // the units that stand for a cell, listed
+            unsigned open = 0xffffffffu;
+#pragma unroll 1
+            for (int round = 0; round < kTilePts; ++round) {  // (every round decides a cell at least)
+                unsigned left = 0u;
+#pragma unroll 1
+                for (int k0 = 0, w0 = tid; w0 - lane < units; k0 += kIn, w0 += kIn * kThreads) {  // warp-uniform
+                    unsigned cn[kIn], won[kIn];
+                    int x[kIn];
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        const int w = w0 + k * kThreads;
+                        cn[k] = (w < units && ((open >> (k0 + k)) & 1u)) ? cell[w] : kNoCell;
+                    }
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        x[k] = -1;
+                        if (cn[k] != kNoCell) {
+                            const int c = kOne ? 0 : (w0 + k * kThreads) / L;
+                            x[k] = word[c * words +
+                                        (ig[c].mode == kCountHash ? __umulhi(cn[k] * mult, ig[c].nslots) : cn[k])];
+                        }
+                    }
+                    int sum = 0;
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        const int w = w0 + k * kThreads;
+                        won[k] = __ballot_sync(0xffffffffu, x[k] == w);
+                        sum += __popc(won[k]);
+                        // (direct words: the index read back is one of the same cell)
+                        if (hashed && x[k] >= 0 && x[k] != w && cell[x[k]] != cn[k]) left |= 1u << (k0 + k);
+                    }
+                    unsigned pos = 0;
+                    if (lane == 0 && sum) pos = atomicAdd(&st.list_n, static_cast<unsigned>(sum));
+                    pos = __shfl_sync(0xffffffffu, pos, 0);
+#pragma unroll
+                    for (int k = 0; k < kIn; ++k) {
+                        if ((won[k] >> lane) & 1u)
+                            list[pos + __popc(won[k] & ((1u << lane) - 1u))] = static_cast<unsigned short>(w0 + k * kThreads);
+                        pos += __popc(won[k]);
+                    }
+                }
+                if (hashed) {
+                    // undecided units (another cell's index in the word): a few go to the
+                    // global table as they are, which settles them exactly; many take
+                    // another round
+                    unsigned pos = 0;
+                    const unsigned cnt = __reduce_add_sync(0xffffffffu, __popc(left));
+                    const unsigned before = warp_incl_scan(static_cast<unsigned>(__popc(left))) - __popc(left);
+                    if (lane == 0 && cnt) pos = atomicAdd(&st.rest_n, cnt);
+                    pos = __shfl_sync(0xffffffffu, pos, 0) + before;
+                    for (unsigned b = left; b; b &= b - 1u, ++pos)
+                        if (pos < kMaxOpen) rest[pos] = static_cast<unsigned short>(tid + (__ffs(b) - 1) * kThreads);
+                }
+                __syncthreads();
+                if (!hashed || st.rest_n <= kMaxOpen) break;
+                __syncthreads();
+                if (tid == 0) st.rest_n = 0u;
+                open = left;
+                mult = mult * 0x85EBCA77u + 0xC2B2AE3Eu;  // (odd again)
+                for (; left; left &= left - 1u) {
+                    const int w = tid + (__ffs(left) - 1) * kThreads;
+                    const int c = kOne ? 0 : w / L;
+                    word[c * words + __umulhi(cell[w] * mult, ig[c].nslots)] = static_cast<unsigned short>(w);
+                }
+                __syncthreads();
+            }
+            const int nl = static_cast<int>(st.list_n);
+            const int nopen = static_cast<int>(st.rest_n);  // (already on the second list)
+            const unsigned short* gl = list;
+            int ng = nl;
+            // (b) a voxel whose every point lies in Morton cells this item holds whole
+            // is counted here (below 256 listed units the test costs about what it saves)
+            if (own && nl >= 256) {
+                unsigned mine = 0;
+                for (int k0 = tid - lane; k0 < nl; k0 += kThreads) {  // warp-uniform
+                    const int k = k0 + lane;
+                    bool glob = false;
+                    int c = 0;
+                    const int w = k < nl ? list[k] : 0;
+                    if (k < nl) {
+                        c = kOne ? 0 : w / L;
+                        const ItemGrid& g = ig[c];
+                        glob = true;
+                        if (g.axis0 >= 0) {
+                            unsigned u[3];
+                            cell_axes(cell[w], g, u);
+                            const unsigned nx = g.bg.nx, ny = static_cast<unsigned>(g.ny);
+                            const uint32_t* t = axis + g.axis0;
+                            const unsigned m = t[u[0]] | t[nx + u[1]] | t[nx + ny + u[2]];
+                            glob = static_cast<int>(m & 0xffffu) < st.own_lo[li] ||
+                                   static_cast<int>(m >> 16) > st.own_hi[li];
+                        }
+                    }
+                    const int pos = warp_append(glob, &st.rest_n);
+                    if (pos >= 0) rest[pos] = static_cast<unsigned short>(w);
+                    if (kOne) mine += (k < nl && !glob) ? 1u : 0u;
+                    else warp_append_keyed(k < nl && !glob, c, st.xcnt);
+                }
+                if (kOne) {
+                    const unsigned t = __reduce_add_sync(0xffffffffu, mine);
+                    if (lane == 0 && t) atomicAdd(&st.xcnt[0], t);
+                }
+                __syncthreads();
+                gl = rest;
+                ng = static_cast<int>(st.rest_n);
+            } else if (nopen) {
+                for (int k = tid; k < nopen; k += kThreads) list[nl + k] = rest[k];
+                __syncthreads();
+                ng = nl + nopen;
+            }
+            // (c) the others into the global tables: a bit per cell of the segment's box
+            // where it fits the table's memory (one round trip, no probing; neighbouring
+            // cells in different slots), else the keys
+            for (int k0 = tid - lane; k0 < ng; k0 += kProbes * kThreads) {  // warp-uniform
+                unsigned long long key[kProbes];
+                unsigned long long* Tp[kProbes];
+                int cc[kProbes];
+                long long slot[kProbes];
+                bool fr[kProbes];
+                bool any_key = false;
+#pragma unroll
+                for (int k2 = 0; k2 < kProbes; ++k2) {
+                    const int k = k0 + lane + k2 * kThreads;
+                    key[k2] = kEmptyKey;
+                    cc[k2] = 0;
+                    slot[k2] = -1;
+                    fr[k2] = false;
+                    if (k < ng) {
+                        const int w = gl[k];
+                        cc[k2] = kOne ? 0 : w / L;
+                        const ItemGrid& g = ig[cc[k2]];
+                        unsigned u[3];
+                        cell_axes(cell[w], g, u);
+#pragma unroll
+                        for (int ax = 0; ax < 3; ++ax) u[ax] += static_cast<unsigned>(g.off[ax]);
+                        Tp[k2] = Tb + cc[k2] * tstride;
+                        if (g.snx) {
+                            const unsigned cell_s = u[0] + g.snx * u[1] + g.snxy * u[2];
+                            slot[k2] = cell_s & ((1u << cap) - 1u);
+                            const unsigned bit = static_cast<unsigned>(static_cast<unsigned long long>(cell_s) >> cap);
+                            const unsigned m = 1u << (bit & 31u);
+                            unsigned* const wd = reinterpret_cast<unsigned*>(Tp[k2] + slot[k2]) + (bit >> 5);
+                            fr[k2] = (atomicAnd(wd, ~m) & m) != 0u;
+                        } else {
+                            key[k2] = static_cast<unsigned long long>(u[0]) | (static_cast<unsigned long long>(u[1]) << 21) |
+                                      (static_cast<unsigned long long>(u[2]) << 42);
+                            any_key = true;
+                        }
+                    } else {
+                        Tp[k2] = Tb;
+                    }
+                }
+                if (any_key) {
+#pragma unroll
+                    for (int k2 = 0; k2 < kProbes; ++k2)
+                        if (key[k2] != kEmptyKey) {
+                            slot[k2] = insert_key(Tp[k2], cap, key[k2]);
+                            if (slot[k2] < 0) bad = HAV_ERR_TABLE_FULL;
+                            fr[k2] = slot[k2] >= 0 && (slot[k2] >> 62);
+                            if (slot[k2] >= 0) slot[k2] &= (1ll << 62) - 1;
+                        }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int k2 = 0; k2 < kProbes; ++k2) log_fresh(slot[k2] >= 0 && fr[k2], cc[k2], slot[k2]);
+            }
+            __syncthreads();
+        }
+        if (bad) {
+            atomicCAS(&sh[s].status, 0, bad);
+            atomicCAS(&gh->status, 0, bad);
+        }
+        if (none) __syncthreads();  // (xcnt and rbits are set)
+        if (ls == nullptr) {  // the count rides on the barrier
+            if (tid == 0) {
+                st.pass_cnt += static_cast<unsigned long long>(st.dcnt[X][li][0]) + st.xcnt[0];
+                if (st.rbits) st.pass_err = 1;
+            }
+        } else {
+            if (tid < ncand && (st.dcnt[X][li][tid] || st.xcnt[tid]))
+                atomicAdd(&ls[s].count[cslot][tid], static_cast<unsigned>(st.dcnt[X][li][tid]) + st.xcnt[tid]);
+            if (tid == 0 && st.rbits) atomicOr(&ls[s].cerr[cslot], st.rbits);
+        }
+        __syncthreads();
+    }
 }
 
 }  // namespace
@@ -455,73 +1081,46 @@ template <int IF, int PR>
 __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_constant__ Plan P) {
     constexpr int kInFlight = PassShape<IF, PR>::kInFlight;
     constexpr int kProbes = PassShape<IF, PR>::kProbes;
-    __shared__ Smem st;
-    extern __shared__ __align__(16) unsigned char dyn[];
+    Smem& st = smem_state();
     const int S = P.S;
     const int tid = threadIdx.x;
     const unsigned nb = static_cast<unsigned>(P.nblocks);
     const long long gtid = static_cast<long long>(blockIdx.x) * kThreads + tid;
     const long long gstride = static_cast<long long>(P.nblocks) * kThreads;
 
-    Dev d;
-    unsigned char* ws = P.ws;
-    d.bar = reinterpret_cast<Barrier*>(ws + P.lay.barrier);
-    d.gh = reinterpret_cast<GlobalHdr*>(ws + P.lay.ghdr);
-    d.sh = reinterpret_cast<SegHdr*>(ws + P.lay.seghdr);
-    d.clean = reinterpret_cast<unsigned*>(ws + P.lay.clean);
-    d.ls = reinterpret_cast<LayerState*>(ws + P.lay.lstate);
-    d.hist = reinterpret_cast<uint32_t*>(ws + P.lay.hist);
-    d.psf = reinterpret_cast<int32_t*>(ws + P.lay.partial_sf);
-    d.pcmp = reinterpret_cast<int32_t*>(ws + P.lay.partial_cmp);
-    d.pitem = reinterpret_cast<int32_t*>(ws + P.lay.pitem);
-    d.tr = reinterpret_cast<hav_layer_trace*>(ws + P.lay.trace);
-    for (int b = 0; b < 2; ++b) {
-        d.ord[b] = reinterpret_cast<float4*>(ws + P.lay.ord[b]);
-        d.orig[b] = reinterpret_cast<int32_t*>(ws + P.lay.orig[b]);
-    d.posof = reinterpret_cast<int32_t*>(ws + P.lay.posof);
-        d.taken[b] = reinterpret_cast<uint32_t*>(ws + P.lay.taken[b]);
-    }
-    for (int b = 0; b < kTableSets; ++b) {
-        d.dirty[b] = reinterpret_cast<uint32_t*>(ws + P.lay.dirty[b]);
-        d.tk[b] = reinterpret_cast<unsigned long long*>(ws + P.lay.tabk[b]);
-    }
-    d.wpre = reinterpret_cast<uint32_t*>(ws + P.lay.wpre);
-    d.bkt = reinterpret_cast<uint32_t*>(ws + P.lay.bkt);
-    d.prefix = reinterpret_cast<int32_t*>(ws + P.lay.prefix);
-    d.tv = reinterpret_cast<unsigned long long*>(ws + P.lay.tabv);
-    d.cand = reinterpret_cast<Cand*>(ws + P.lay.cand);
-    d.ptimes = P.ptimes;
-    d.ptimes_cap = P.ptimes_cap;
+    const Dev d{P};
+#pragma unroll 1
     for (int k = tid; k < P.S; k += kThreads) st.gm[k] = 0;  // no previous search yet
     if (tid == 0) st.bucketed = 0;
     if (tid == 0) {
         st.fused_uses[0] = st.fused_uses[1] = 0u;
         st.fused_last[0] = st.fused_last[1] = 0ull;
         st.epoch = 0u;
-        st.set_clean = 0;
         st.ntimes = 0;
         // every block reads this before block 0 may change it (after the first barrier)
-        st.was_clean = static_cast<int>(ld_volatile_u(d.clean));
-        if (d.ptimes && blockIdx.x == 0) {
-            d.ptimes[0] = globaltimer();
-            d.ptimes[1] = 0;
+        st.was_clean = static_cast<int>(ld_volatile_u(d.clean()));
+        if (d.ptimes() && blockIdx.x == 0) {
+            d.ptimes()[0] = globaltimer();
+            d.ptimes()[1] = 0;
             st.ntimes = 1;
         }
     }
     __syncthreads();
 
+#pragma unroll 1
     for (int j = 0; j < P.L; ++j) {
         level_setup(P, j, st);
         if (tid < kLocalItems) st.own_on[tid] = 0;
-        float4* ord = d.ord[j & 1];
-        const int32_t* orig_in = (j == 0) ? nullptr : d.orig[(j - 1) & 1];
-        uint32_t* taken = d.taken[j & 1];
+        float4* ord = d.ord(j & 1);
+        const int32_t* orig_in = (j == 0) ? nullptr : d.orig((j - 1) & 1);
+        uint32_t* taken = d.taken(j & 1);
         const long long NL = st.n_level;
         // level 0: every segment of at least kBucketMin points is sorted by
         // Morton cell (one cloud: the whole level; a batch: each such segment
         // within its own range)
         bool bucketing = false;
         if (j == 0)
+#pragma unroll 1
             for (int s2 = 0; s2 < S; ++s2) bucketing = bucketing || st.n[s2] >= kBucketMin;
 
         // ------------------------------------------------ bbox, layout, clears
@@ -529,27 +1128,17 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
         // level's compaction, which wrote its points)
         if (j == 0) {
             const int par = j & 1;
+#pragma unroll 1
             for (int it = blockIdx.x; it < st.items_total; it += nb) {
                 int a, b;
                 const int s = item_range(st, S, it, &a, &b);
                 float mnv[3] = {INFINITY, INFINITY, INFINITY}, mxv[3] = {-INFINITY, -INFINITY, -INFINITY};
                 int bad = 0;
-                for (int i = a + tid; i < b; i += kThreads) {
-                    float p[3];
-                    if (j == 0) {
-                        const float* q = P.points + 3 * i;
-                        p[0] = q[0];
-                        p[1] = q[1];
-                        p[2] = q[2];
-                        if (st.n[s] < kBucketMin) {  // (a bucketed segment is placed by its scatter)
-                            ord[i] = make_float4(p[0], p[1], p[2], __int_as_float(static_cast<int>(i)));
-                            d.posof[i] = static_cast<int32_t>(i);
-                        }
-                    } else {
-                        const float4 q = ord[i];
-                        p[0] = q.x;
-                        p[1] = q.y;
-                        p[2] = q.z;
+                const bool place = st.n[s] < kBucketMin;  // (a bucketed segment is placed by its scatter)
+                for_points(P.points, a, b, [&](int i, const float* p) {
+                    if (place) {
+                        ord[i] = make_float4(p[0], p[1], p[2], __int_as_float(i));
+                        d.posof()[i] = i;
                     }
 #pragma unroll
                     for (int a3 = 0; a3 < 3; ++a3) {
@@ -557,9 +1146,10 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                         mnv[a3] = fminf(mnv[a3], p[a3]);
                         mxv[a3] = fmaxf(mxv[a3], p[a3]);
                     }
-                }
+                });
 #pragma unroll
                 for (int a3 = 0; a3 < 3; ++a3) {
+#pragma unroll 1
                     for (int o = 16; o > 0; o >>= 1) {
                         mnv[a3] = fminf(mnv[a3], __shfl_xor_sync(0xffffffffu, mnv[a3], o));
                         mxv[a3] = fmaxf(mxv[a3], __shfl_xor_sync(0xffffffffu, mxv[a3], o));
@@ -574,34 +1164,36 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 bad = __syncthreads_or(bad);
                 if (tid < 6) {
                     float r = st.redf[tid][0];
+#pragma unroll 1
                     for (int w = 1; w < kThreads / 32; ++w)
                         r = (tid < 3) ? fminf(r, st.redf[tid][w]) : fmaxf(r, st.redf[tid][w]);
                     if (isfinite(r)) {
-                        if (tid < 3) atomicMax(&d.sh[s].bbox[par][tid], ~enc_f(r));
-                        else atomicMax(&d.sh[s].bbox[par][tid], enc_f(r));
+                        if (tid < 3) atomicMax(&d.sh()[s].bbox[par][tid], ~enc_f(r));
+                        else atomicMax(&d.sh()[s].bbox[par][tid], enc_f(r));
                     }
                 }
                 if (tid == 0 && bad) {
-                    atomicExch(&d.sh[s].nonfinite, 1);
+                    atomicExch(&d.sh()[s].nonfinite, 1);
                     seg_error(d, s, HAV_ERR_NONFINITE);
                 }
                 __syncthreads();
             }
             fill<uint32_t>(taken, NL / 32 + 1, 0u, gtid, gstride);
-            fill<int32_t>(d.prefix, static_cast<long long>(S) * kMaxIters, -1, gtid, gstride);
+            fill<int32_t>(d.prefix(), static_cast<long long>(S) * kMaxIters, -1, gtid, gstride);
             clear_layer_state(d, S, 0, gtid, gstride);
             clear_layer_state(d, S, 1, gtid, gstride);
             if (j == 0 && !st.was_clean) {
                 // first call on this workspace, or the previous call was cut short
+#pragma unroll 1
                 for (int b = 0; b < kTableSets; ++b)
-                    fill<unsigned long long>(d.tk[b], P.lay.tab_slots, kEmptyKey, gtid, gstride);
-                fill<unsigned long long>(d.tv, P.lay.tab_slots, kEmptyVal, gtid, gstride);
+                    fill<unsigned long long>(d.tk(b), P.lay.tab_slots, kEmptyKey, gtid, gstride);
+                fill<unsigned long long>(d.tv(), P.lay.tab_slots, kEmptyVal, gtid, gstride);
             }
-            if (bucketing) fill<uint32_t>(d.bkt, 2 * 4096ll * S, 0u, gtid, gstride);
+            if (bucketing) fill<uint32_t>(d.bkt(), 2 * 4096ll * S, 0u, gtid, gstride);
             // (test hook: one arrival more than the launch has blocks never comes,
             // so every block's bounded wait gives up and the call reports a timeout)
             if (!grid_sync(d, nb + ((j == 0 && P.test_timeout) ? 1u : 0u), st, TAG(1, j, 0, 0))) return;
-            if (j == 0 && blockIdx.x == 0 && tid == 0) *(volatile unsigned*)d.clean = 0u;
+            if (j == 0 && blockIdx.x == 0 && tid == 0) *(volatile unsigned*)d.clean() = 0u;
         }
 
         // --------------------------------------------------- search bracket
@@ -611,11 +1203,11 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             // others read them: the error carried from the previous level's
             // compaction, and the non-finite flag of this level's bbox phase
             int err = (j == 0) ? 0 : st.err[tid];
-            if (!err && ld_volatile(&d.sh[tid].nonfinite)) err = HAV_ERR_NONFINITE;
+            if (!err && ld_volatile(&d.sh()[tid].nonfinite)) err = HAV_ERR_NONFINITE;
             float s_hi = 0.0f;
             for (int a = 0; a < 3; ++a) {
-                float mn = dec_f(~d.sh[tid].bbox[par][a]);
-                float mx = dec_f(d.sh[tid].bbox[par][3 + a]);
+                float mn = dec_f(~d.sh()[tid].bbox[par][a]);
+                float mx = dec_f(d.sh()[tid].bbox[par][3 + a]);
                 if (st.n[tid] == 0 || err) mn = mx = 0.0f;
                 st.mn[tid][a] = mn;
                 st.mx[tid][a] = mx;
@@ -645,11 +1237,11 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             const int li = tid;
             int ia, ib;
             const int s = item_range(st, S, static_cast<int>(blockIdx.x + tid * nb), &ia, &ib);
-            if (ld_volatile(&d.sh[s].b0_on) && ib > ia) {
+            if (ld_volatile(&d.sh()[s].b0_on) && ib > ia) {
                 float mn3[3], mx3[3], k3[3];
                 for (int a3 = 0; a3 < 3; ++a3) {
-                    mn3[a3] = d.sh[s].b0[a3];
-                    mx3[a3] = d.sh[s].b0[3 + a3];
+                    mn3[a3] = d.sh()[s].b0[a3];
+                    mx3[a3] = d.sh()[s].b0[3 + a3];
                     const float e = __fsub_rn(mx3[a3], mn3[a3]);
                     k3[a3] = (e > 0.0f) ? __fdiv_rn(16.0f, e) : 0.0f;
                 }
@@ -698,23 +1290,22 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
 
         // ---------------------------------------- bucketing (one large cloud)
         if (bucketing && S == 1) {
-            if (tid == 0) st.set_clean = 0;
             uint32_t* h = reinterpret_cast<uint32_t*>(dyn);          // this block's counts
             uint32_t* hb = reinterpret_cast<uint32_t*>(dyn) + 4096;  // global bucket bases
+#pragma unroll 1
             for (int b = tid; b < 4096; b += kThreads) h[b] = 0u;
             __syncthreads();
+#pragma unroll 1
             for (int it = blockIdx.x; it < st.items_total; it += nb) {
                 int a, b;
                 item_range(st, S, it, &a, &b);
-                for (int i = a + tid; i < b; i += kThreads) {
-                    const float* q = P.points + 3 * i;
-                    const float p[3] = {q[0], q[1], q[2]};
-                    atomicAdd(&h[bucket_of(p, st.mn[0], st.mx[0])], 1u);
-                }
+                for_points(P.points, a, b,
+                           [&](int, const float* p) { atomicAdd(&h[bucket_of(p, st.mn[0], st.mx[0])], 1u); });
             }
             __syncthreads();
+#pragma unroll 1
             for (int b = tid; b < 4096; b += kThreads)
-                if (h[b]) atomicAdd(&d.bkt[b], h[b]);
+                if (h[b]) atomicAdd(&d.bkt()[b], h[b]);
             if (!grid_sync(d, nb, st, TAG(9, j, 0, 0))) return;
             {
                 // exclusive prefix over the 4096 global counts (whole bins per thread)
@@ -723,7 +1314,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 uint32_t c4[kPerT], sum = 0;
 #pragma unroll
                 for (int k = 0; k < kPerT; ++k) {
-                    c4[k] = d.bkt[kPerT * tid + k];
+                    c4[k] = d.bkt()[kPerT * tid + k];
                     sum += c4[k];
                 }
                 unsigned tot;
@@ -754,21 +1345,21 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     item_range(st, S, static_cast<int>(blockIdx.x + tid * nb), &ia, &ib);
                     own_cells(hb, ia, ib, static_cast<unsigned>(NL), st.b0_mn, st.b0_k, st, tid);
                 }
+#pragma unroll 1
                 for (int b = tid; b < 4096; b += kThreads)
-                    if (h[b]) h[b] = hb[b] + atomicAdd(&d.bkt[4096 + b], h[b]);
+                    if (h[b]) h[b] = hb[b] + atomicAdd(&d.bkt()[4096 + b], h[b]);
                 __syncthreads();
+#pragma unroll 1
                 for (int it = blockIdx.x; it < st.items_total; it += nb) {
                     int a, b;
                     item_range(st, S, it, &a, &b);
-                    for (int i = a + tid; i < b; i += kThreads) {
-                        const float* q = P.points + 3 * i;
-                        const float p[3] = {q[0], q[1], q[2]};
+                    for_points(P.points, a, b, [&](int i, const float* p) {
                         const unsigned r = atomicAdd(&h[bucket_of(p, st.mn[0], st.mx[0])], 1u);
                         if (r < static_cast<unsigned>(NL)) {
-                            ord[r] = make_float4(p[0], p[1], p[2], __int_as_float(static_cast<int>(i)));
-                            d.posof[i] = static_cast<int32_t>(r);
+                            ord[r] = make_float4(p[0], p[1], p[2], __int_as_float(i));
+                            d.posof()[i] = static_cast<int32_t>(r);
                         }
-                    }
+                    });
                 }
             }
             if (!grid_sync(d, nb, st, TAG(10, j, 0, 0))) return;
@@ -783,28 +1374,31 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             // phase.  (Leaving a segment that comes in a coherent order, a
             // LiDAR scan, unsorted measured 0.9 % slower on 64 LiDAR clouds:
             // the ownership test needs the sort.)
-            if (tid == 0) st.set_clean = 0;
             uint32_t* h = reinterpret_cast<uint32_t*>(dyn);          // counts of one segment's items
             uint32_t* hb = reinterpret_cast<uint32_t*>(dyn) + 4096;  // bases of one segment's buckets
-            uint32_t* bcnt = d.bkt;
-            uint32_t* bcur = d.bkt + 4096ll * S;
+            uint32_t* bcnt = d.bkt();
+            uint32_t* bcur = d.bkt() + 4096ll * S;
             if (blockIdx.x == 0)  // the boxes of the sorted segments, for their later levels
+#pragma unroll 1
                 for (int s2 = tid; s2 < S; s2 += kThreads)
                     if (st.n[s2] >= kBucketMin) {
                         for (int a3 = 0; a3 < 3; ++a3) {
-                            d.sh[s2].b0[a3] = st.mn[s2][a3];
-                            d.sh[s2].b0[3 + a3] = st.mx[s2][a3];
+                            d.sh()[s2].b0[a3] = st.mn[s2][a3];
+                            d.sh()[s2].b0[3 + a3] = st.mx[s2][a3];
                         }
-                        d.sh[s2].b0_on = 1;
+                        d.sh()[s2].b0_on = 1;
                     }
             int hs = -1;  // the segment whose counts h holds
+#pragma unroll 1
             for (int b = tid; b < 4096; b += kThreads) h[b] = 0u;
             __syncthreads();
+#pragma unroll 1
             for (int it = blockIdx.x; it < st.items_total; it += nb) {  // (block-uniform)
                 int a, b;
                 const int s = item_range(st, S, it, &a, &b);
                 if (st.n[s] < kBucketMin) continue;
                 if (hs >= 0 && hs != s) {
+#pragma unroll 1
                     for (int k = tid; k < 4096; k += kThreads)
                         if (h[k]) {
                             atomicAdd(&bcnt[4096ll * hs + k], h[k]);
@@ -813,18 +1407,17 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     __syncthreads();
                 }
                 hs = s;
-                for (int i = a + tid; i < b; i += kThreads) {
-                    const float* q = P.points + 3 * i;
-                    const float p3[3] = {q[0], q[1], q[2]};
-                    atomicAdd(&h[bucket_of(p3, st.mn[s], st.mx[s])], 1u);
-                }
+                for_points(P.points, a, b,
+                           [&](int, const float* p3) { atomicAdd(&h[bucket_of(p3, st.mn[s], st.mx[s])], 1u); });
                 __syncthreads();
             }
             if (hs >= 0)
+#pragma unroll 1
                 for (int k = tid; k < 4096; k += kThreads)
                     if (h[k]) atomicAdd(&bcnt[4096ll * hs + k], h[k]);
             if (!grid_sync(d, nb, st, TAG(9, j, 0, 0))) return;
             int bs = -1;  // the segment whose bases hb holds
+#pragma unroll 1
             for (int it = blockIdx.x; it < st.items_total; it += nb) {  // (block-uniform)
                 int a, b;
                 const int s = item_range(st, S, it, &a, &b);
@@ -848,6 +1441,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     }
                     bs = s;
                 }
+#pragma unroll 1
                 for (int k = tid; k < 4096; k += kThreads) h[k] = 0u;
                 __syncthreads();
                 if (tid == 0) {  // the cells this item holds whole, in its segment's box
@@ -858,39 +1452,38 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     }
                     own_cells(hb, a, b, static_cast<unsigned>(st.off[s + 1]), st.mn[s], k3, st, li);
                 }
-                for (int i = a + tid; i < b; i += kThreads) {
-                    const float* q = P.points + 3 * i;
-                    const float p3[3] = {q[0], q[1], q[2]};
-                    atomicAdd(&h[bucket_of(p3, st.mn[s], st.mx[s])], 1u);
-                }
+                for_points(P.points, a, b,
+                           [&](int, const float* p3) { atomicAdd(&h[bucket_of(p3, st.mn[s], st.mx[s])], 1u); });
                 __syncthreads();
+#pragma unroll 1
                 for (int k = tid; k < 4096; k += kThreads)
                     if (h[k]) h[k] = hb[k] + atomicAdd(&bcur[4096ll * s + k], h[k]);
                 __syncthreads();
                 const unsigned end = static_cast<unsigned>(st.off[s + 1]);
-                for (int i = a + tid; i < b; i += kThreads) {
-                    const float* q = P.points + 3 * i;
-                    const float p3[3] = {q[0], q[1], q[2]};
+                for_points(P.points, a, b, [&](int i, const float* p3) {
                     const unsigned r = atomicAdd(&h[bucket_of(p3, st.mn[s], st.mx[s])], 1u);
                     if (r < end) {
-                        ord[r] = make_float4(p3[0], p3[1], p3[2], __int_as_float(static_cast<int>(i)));
-                        d.posof[i] = static_cast<int32_t>(r);
+                        ord[r] = make_float4(p3[0], p3[1], p3[2], __int_as_float(i));
+                        d.posof()[i] = static_cast<int32_t>(r);
                     }
-                }
+                });
                 __syncthreads();
             }
             if (!grid_sync(d, nb, st, TAG(10, j, 0, 0))) return;
         }
+
+        item_boxes(S, nb, ord);
 
         // ------------------------------------------------------------ layers
         long long taken_before = 0;  // thread s: budgets of earlier layers of segment s
         const int ncand = st.ncand;
         const long long tstride = st.tab_stride;  // table slots of one candidate (all segments)
         const long long dstride = NL;             // log entries of one candidate
+#pragma unroll 1
         for (int l = 0; l < P.layers; ++l) {
             const int q = l & 1;
-            LayerState* ls = d.ls + q * S;
-            uint32_t* hist = d.hist + static_cast<long long>(q) * S * kHistBins;
+            LayerState* ls = d.ls() + q * S;
+            uint32_t* hist = d.hist() + static_cast<long long>(q) * S * kHistBins;
 
             if (tid < S) {
                 const long long ml = layer_budget(st.m[tid], P.layers, P.ratio, l);
@@ -931,7 +1524,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 }
                 st.flags[tid] = fl;
                 if (blockIdx.x == 0) {
-                    hav_layer_trace* tr = d.tr + (static_cast<long long>(j) * S + tid) * kMaxLayers + l;
+                    hav_layer_trace* tr = d.tr() + (static_cast<long long>(j) * S + tid) * kMaxLayers + l;
                     tr->m_l = ml;
                     tr->k_max = kmax;
                     tr->k_star = 0;
@@ -954,15 +1547,17 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             if (P.search == HAV_SEARCH_BISECT && P.t_max > 0) {
                 static_assert(kMaxIters <= 32, "one lane per step");
                 const int lane = tid & 31;
+#pragma unroll 1
                 for (int s = tid >> 5; s < S; s += kThreads / 32) {  // (warp-uniform)
                     if (!(st.flags[s] & F_SEARCH)) continue;
                     const long long ml = st.ml[s];
                     float sv = st.s_hi[s];
+#pragma unroll 1
                     for (int h = 0; h <= lane; ++h) sv = __fmul_rn(__fadd_rn(0.0f, sv), 0.5f);
                     long long bd = LLONG_MAX;
                     if (lane < P.t_max) {
                         bd = cell_bound(sv, P.aspect, st.mn[s], st.mx[s]);
-                        const int pk = ld_volatile(d.prefix + s * kMaxIters + lane);
+                        const int pk = ld_volatile(d.prefix() + s * kMaxIters + lane);
                         if (pk >= 0 && pk < bd) bd = pk;
                     }
                     const unsigned settled = __ballot_sync(0xffffffffu, lane < P.t_max && bd < ml);
@@ -985,7 +1580,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                         st.flags[s] = fl;
                     }
                     if (blockIdx.x == 0) {
-                        hav_layer_trace* tr = d.tr + (static_cast<long long>(j) * S + s) * kMaxLayers + l;
+                        hav_layer_trace* tr = d.tr() + (static_cast<long long>(j) * S + s) * kMaxLayers + l;
                         if (lane < nskip) {
                             tr->s[lane] = sv;
                             tr->K[lane] = bd;
@@ -1009,6 +1604,11 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             // plain bisection; D = 1 is the plain bisection.
             // one cloud, one candidate per pass: the count rides on the barrier
             const bool fused = (S == 1 && ncand == 1);
+            // the next pass's grids, for every outcome of this one, are prepared while
+            // the other blocks arrive, where they fit
+            const int my_items = (st.items_total - static_cast<int>(blockIdx.x) + static_cast<int>(nb) - 1) / static_cast<int>(nb);
+            const bool ahead = my_items * (ncand + 1) * ncand <= kPassGrids;
+#pragma unroll 1
             for (int p = 0; p < P.t_max; ++p) {
                 const int searching = (tid < S && (st.flags[tid] & F_SEARCH)) ? 1 : 0;
                 if (tid == 0) {
@@ -1022,181 +1622,21 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 const int Z = (p + kTableSets - 1) % kTableSets;
                 const int F = (p + 1) % kTableSets;
 
-                // candidate grids of the owned items' segments
                 {
-                    int li = 0;
-                    for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
-                        const int s = find_seg(st.item0, S, it);
-                        if (tid < ncand && (st.flags[s] & F_SEARCH)) {
-                            const float sc = cand_size(st.lo[s], st.hi[s], (st.flags[s] & F_UP) != 0,
-                                                       st.first[s], tid);
-                            st.cvalid[li][tid] = make_grid(sc, P.aspect, st.mn[s], &st.cgrid[li][tid]) ? 1 : 0;
-                        }
-                    }
-                }
-                __syncthreads();
-
-                // Cnt(P_l, s_c) for every candidate c: (a) every point's key into the
-                // candidate's part of the block set, keys new to the block listed
-                // densely; (b) the listed keys into the candidates' global tables,
-                // kProbes compare-and-swaps in flight per thread
-                unsigned long long* set = reinterpret_cast<unsigned long long*>(dyn);
-                unsigned short* list = reinterpret_cast<unsigned short*>(dyn + kSetSlots * sizeof(unsigned long long));
-                const int setc_log2 = st.setc_log2;
-                int li = 0;
-                for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
-                    int a, b;
-                    const int s = item_range(st, S, it, &a, &b);
-                    if (!(st.flags[s] & F_SEARCH)) continue;
-                    if (!st.set_clean)  // otherwise every slot is already empty
-                        for (int k = tid; k < kSetSlots; k += kThreads) set[k] = kEmptyKey;
-                    if (tid == 0) {
-                        st.list_n = 0u;
-                        st.rbits = 0u;
-                        st.rest_n = 0u;
-                    }
-                    if (tid < kMaxCand) st.xcnt[tid] = 0u;
-                    __syncthreads();
-                    const int cap = st.cap_log2[s];
-                    unsigned long long* Tb = d.tk[X] + st.tab_off[s];
-                    int bad = 0;
-                    unsigned rbits = 0;  // candidates with a key out of range
-                    // log a fresh insert (whole warp calls, converged): one shared
-                    // counter add per candidate present in the warp, and the warp's
-                    // log entries of a candidate land side by side.  The set X logs
-                    // are empty when a pass starts, so dcnt[X] ends as the count.
-                    auto log_fresh = [&](bool fresh, int c, long long slot) {
-                        const int k = (ncand == 1) ? warp_append(fresh, &st.dcnt[X][li][0])
-                                                   : warp_append_keyed(fresh, c, st.dcnt[X][li]);
-                        if (fresh)
-                            d.dirty[X][c * dstride + a + k] = static_cast<uint32_t>(c * tstride + st.tab_off[s] + slot);
-                    };
-                    // work units are (candidate, point) pairs, point-minor, so that a
-                    // warp reads consecutive points and the candidates run in parallel
-                    const int lane = tid & 31;
-                    const int L = b - a;
-                    const int units = L * ncand;
-                    for (int base = tid - lane; base < units; base += kInFlight * kThreads) {  // warp-uniform
-                        float4 q4[kInFlight];
-                        int cu[kInFlight];
-#pragma unroll
-                        for (int u = 0; u < kInFlight; ++u) {
-                            const int w = base + lane + u * kThreads;
-                            cu[u] = (ncand == 1) ? 0 : w / L;
-                            q4[u] = (w < units) ? ord[a + (w - cu[u] * L)]
-                                                : make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-                        }
-                        // the keys of all units first (independent arithmetic), then
-                        // their inserts one after the other
-                        unsigned long long key[kInFlight];
-#pragma unroll
-                        for (int u = 0; u < kInFlight; ++u) {
-                            key[u] = kEmptyKey;
-                            const int c = cu[u];
-                            // w < 0: padding, or taken by an earlier layer
-                            if (__float_as_int(q4[u].w) >= 0 && st.cvalid[li][c]) {
-                                const float p3[3] = {q4[u].x, q4[u].y, q4[u].z};
-                                float f[3];
-                                if (!cell_key(p3, st.cgrid[li][c], &key[u], f)) {
-                                    rbits |= 1u << c;
-                                    key[u] = kEmptyKey;
-                                }
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < kInFlight; ++u) {
-                            const int c = cu[u];
-                            int r = -2;
-                            bool nw = false;
-                            if (key[u] != kEmptyKey) r = smem_insert_n(set + (c << setc_log2), setc_log2, key[u], &nw);
-                            const int pos = warp_append(r >= 0 && nw, &st.list_n);
-                            if (pos >= 0) list[pos] = static_cast<unsigned short>((c << setc_log2) + r);
-                            bool fr = false;
-                            long long slot = -1;
-                            if (r == -1) {  // block set saturated: straight to the global table
-                                slot = find_or_insert(Tb + c * tstride, cap, key[u], &fr);
-                                if (slot < 0) bad = HAV_ERR_TABLE_FULL;
-                            }
-                            log_fresh(r == -1 && slot >= 0 && fr, c, slot);
-                        }
-                    }
-                    __syncthreads();
-                    const int nl = static_cast<int>(st.list_n);
-                    // a voxel whose every point lies in cells this block holds
-                    // whole is counted here; the other keys go to the global table
-                    const unsigned short* gl = list;
-                    int ng = nl;
-                    // (below 256 listed keys the test costs about what it saves)
-                    if (st.own_on[li] && nl >= 256 && nl <= kSetSlots / 2) {
-                        unsigned short* rest = list + kSetSlots / 2;
-                        unsigned mine = 0;  // owned keys of this thread (one candidate)
-                        for (int k0 = tid - lane; k0 < nl; k0 += kThreads) {  // warp-uniform
-                            const int k = k0 + lane;
-                            bool glob = false;
-                            int c = 0;
-                            if (k < nl) {
-                                const int idx = list[k];
-                                c = idx >> setc_log2;
-                                glob = !voxel_owned(set[idx], st.cgrid[li][c], st.own_mn[li], st.own_k[li],
-                                                    st.own_lo[li], st.own_hi[li]);
-                            }
-                            const int pos = warp_append(glob, &st.rest_n);
-                            if (pos >= 0) rest[pos] = list[k];
-                            if (ncand == 1) mine += (k < nl && !glob) ? 1u : 0u;
-                            else warp_append_keyed(k < nl && !glob, c, st.xcnt);
-                        }
-                        if (ncand == 1) {
-                            const unsigned w = __reduce_add_sync(0xffffffffu, mine);
-                            if (lane == 0 && w) atomicAdd(&st.xcnt[0], w);
-                        }
-                        __syncthreads();
-                        gl = rest;
-                        ng = static_cast<int>(st.rest_n);
-                    }
-                    for (int k0 = tid - lane; k0 < ng; k0 += kProbes * kThreads) {  // warp-uniform
-                        unsigned long long key[kProbes];
-                        unsigned long long* Tp[kProbes];
-                        int cc[kProbes];
-                        long long slot[kProbes];
-                        bool fr[kProbes];
-#pragma unroll
-                        for (int u = 0; u < kProbes; ++u) {
-                            const int k = k0 + lane + u * kThreads;
-                            const int idx = (k < ng) ? static_cast<int>(gl[k]) : 0;
-                            cc[u] = idx >> setc_log2;
-                            key[u] = (k < ng) ? set[idx] : kEmptyKey;
-                            Tp[u] = Tb + cc[u] * tstride;
-                        }
-                        find_or_insert_batch<kProbes>(Tp, cap, key, slot, fr);
-#pragma unroll
-                        for (int u = 0; u < kProbes; ++u) {
-                            if (key[u] != kEmptyKey && slot[u] < 0) bad = HAV_ERR_TABLE_FULL;
-                            log_fresh(key[u] != kEmptyKey && slot[u] >= 0 && fr[u], cc[u], slot[u]);
-                        }
-                    }
-                    // empty the set again: exactly the listed slots are occupied
-                    __syncthreads();
-                    for (int k = tid; k < nl; k += kThreads) set[list[k]] = kEmptyKey;
-                    if (tid == 0) st.set_clean = 1;
-                    if (rbits) atomicOr(&st.rbits, rbits);
-                    if (bad) seg_error(d, s, bad);
-                    __syncthreads();
-                    if (fused) {
-                        if (tid == 0) {
-                            st.pass_cnt += static_cast<unsigned long long>(st.dcnt[X][li][0]) + st.xcnt[0];
-                            if (st.rbits) st.pass_err = 1;
-                        }
-                    } else {
-                        if (tid < ncand && (st.dcnt[X][li][tid] || st.xcnt[tid]))
-                            atomicAdd(&ls[s].count[p % 3][tid], static_cast<unsigned>(st.dcnt[X][li][tid]) + st.xcnt[tid]);
-                        if (tid == 0 && st.rbits) atomicOr(&ls[s].cerr[p % 3], st.rbits);
-                    }
+                    LayerState* const pls = fused ? nullptr : ls;
+                    if (ncand == 1)
+                        pass_items<kProbes, true>(S, nb, ord, d.tk(X), d.dirty(X), X, dstride, pls, p % 3, d.sh(), d.gh(),
+                                                  ahead && p > 0, P.aspect[0], P.aspect[1], P.aspect[2]);
+                    else
+                        pass_items<kProbes, false>(S, nb, ord, d.tk(X), d.dirty(X), X, dstride, pls, p % 3, d.sh(), d.gh(),
+                                                   ahead && p > 0, P.aspect[0], P.aspect[1], P.aspect[2]);
                 }
                 if (fused) {
                     const unsigned long long add = st.pass_cnt + (st.pass_err ? kFusedErr : 0ull);
                     fused_arrive(d, st, p & 1, add);
                 } else {
                     if (p >= 1 && blockIdx.x == 0)
+#pragma unroll 1
                         for (int k = tid; k < S * (kMaxCand + 1); k += kThreads) {
                             const int s = k / (kMaxCand + 1), c = k % (kMaxCand + 1);
                             if (c < kMaxCand) ls[s].count[(p + 1) % 3][c] = 0u;
@@ -1210,23 +1650,29 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 // publishes the stores, before pass p + 2 inserts into set Z.
                 if (p >= 1) {
                     int li = 0;
+#pragma unroll 1
                     for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
                         int a, b;
                         const int s = item_range(st, S, it, &a, &b);
                         if (!(st.flags[s] & F_SEARCH)) continue;
+#pragma unroll 1
                         for (int c = 0; c < ncand; ++c) {
                             const int cnt = st.dcnt[Z][li][c];
-                            const uint32_t* lg = d.dirty[Z] + c * dstride + a;
-                            for (int k = tid; k < cnt; k += kThreads) d.tk[Z][lg[k]] = kEmptyKey;
+                            const uint32_t* lg = d.dirty(Z) + c * dstride + a;
+#pragma unroll 4
+                            for (int k = tid; k < cnt; k += kThreads) d.tk(Z)[lg[k]] = kEmptyKey;
                         }
                     }
                     __syncthreads();
                     li = 0;
+#pragma unroll 1
                     for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
                         const int s = find_seg(st.item0, S, it);
                         if (tid < ncand && (st.flags[s] & F_SEARCH)) st.dcnt[Z][li][tid] = 0;
                     }
                 }
+                if (ahead && my_items > 0)
+                    item_grids(S, nb, 1, 0, my_items * (ncand + 1) * ncand, ncand + 1, P.aspect[0], P.aspect[1], P.aspect[2]);
                 if (fused) {
                     if (!fused_wait(d, nb, st, p & 1, TAG(2, j, l, p))) return;
                 } else {
@@ -1248,12 +1694,19 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
 #pragma unroll
                     for (int c = 0; c < kMaxCand; ++c)
                         cnt[c] = (!fused && c < ncand) ? ld_volatile_u(&ls[tid].count[p % 3][c]) : 0u;
-                    hav_layer_trace* tr = d.tr + (static_cast<long long>(j) * S + tid) * kMaxLayers + l;
+                    hav_layer_trace* tr = d.tr() + (static_cast<long long>(j) * S + tid) * kMaxLayers + l;
                     while (node < ncand && t < P.t_max) {
                         const float sv = next_size(lo, hi, up, first);
                         first = 0.0f;
+                        // (sizes well inside the range need no grid to be known representable)
+                        bool fine = !((cerr >> node) & 1u);
+                        for (int a = 0; a < 3; ++a) {
+                            const float v = __fmul_rn(sv, P.aspect[a]);
+                            fine = fine && v > 7.8886090522101181e-31f && v < 1.2676506002282294e30f &&
+                                   fabsf(st.mn[tid][a]) < __fmul_rn(v, 1.0e18f);
+                        }
                         Grid gv;
-                        if ((cerr >> node) & 1u || !make_grid(sv, P.aspect, st.mn[tid], &gv)) {
+                        if (!fine && (((cerr >> node) & 1u) || !make_grid(sv, P.aspect, st.mn[tid], &gv))) {
                             seg_error(d, tid, HAV_ERR_RANGE);
                             st.err[tid] = HAV_ERR_RANGE;
                             st.flags[tid] = 0;
@@ -1270,7 +1723,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                             tr->iters = t + 1;
                         }
                         if (pre) {  // sv = s_hi / 2^(t+1): later layers of the level may reuse K
-                            if (blockIdx.x == 0) d.prefix[tid * kMaxIters + t] = static_cast<int32_t>(K);
+                            if (blockIdx.x == 0) d.prefix()[tid * kMaxIters + t] = static_cast<int32_t>(K);
                             if (K >= st.ml[tid]) pre = false;
                         }
                         ++t;
@@ -1282,14 +1735,17 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                             up = false;
                             node = 2 * node + 1;
                         } else {
+                            // (the selection's keys go to set F, empty for this segment: the
+                            // pass's own table may hold bits)
                             st.s_star[tid] = sv;
-                            st.grid[tid] = gv;
-                            st.sel[tid] = X;
-                            st.sel_cand[tid] = node;
+                            make_grid(sv, P.aspect, st.mn[tid], &st.grid[tid]);
+                            st.sel[tid] = F;
+                            st.sel_cand[tid] = 0;
                             st.flags[tid] = F_ACTIVE | F_ACCEPT;
                             break;
                         }
                     }
+                    st.leaf[tid] = node - ncand;  // (a search that goes on has walked to a leaf)
                     st.lo[tid] = lo;
                     st.hi[tid] = hi;
                     st.iters[tid] = t;
@@ -1321,26 +1777,28 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 st.gs[tid] = st.s_star[tid];
                 st.gm[tid] = st.ml[tid];
                 if (blockIdx.x == 0) {  // for a small-level launch that continues the chain
-                    d.sh[tid].guide_s = st.gs[tid];
-                    d.sh[tid].guide_m = st.gm[tid];
+                    d.sh()[tid].guide_s = st.gs[tid];
+                    d.sh()[tid].guide_m = st.gm[tid];
                 }
             }
 
             // ------------------------------------- Section 3.2 selection at s*
             {
-                if (tid == 0) st.set_clean = 0;
                 unsigned long long* skey = reinterpret_cast<unsigned long long*>(dyn);
                 unsigned long long* sval = skey + kSelSlots;
                 unsigned short* list = reinterpret_cast<unsigned short*>(sval + kSelSlots);
                 int li = 0;
+#pragma unroll 1
                 for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
                     int a, b;
                     const int s = item_range(st, S, it, &a, &b);
                     if (!(st.flags[s] & F_ACTIVE)) continue;
+#pragma unroll 1
                     for (int k = tid; k < kSelSlots; k += kThreads) {
                         skey[k] = kEmptyKey;
                         sval[k] = kEmptyVal;
                     }
+#pragma unroll 1
                     for (int k = tid; k < kHistBins; k += kThreads) st.bh[k] = 0u;
                     if (tid == 0) {
                         st.list_n = 0u;
@@ -1354,18 +1812,18 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     // table and is listed for the classification (in the next level's
                     // staged-point array, not written before this level's compaction)
                     const bool owning = st.own_on[li] != 0;
-                    Cand* olist = reinterpret_cast<Cand*>(d.ord[(j + 1) & 1]) + a;
+                    Cand* olist = reinterpret_cast<Cand*>(d.ord((j + 1) & 1)) + a;
                     const int sel = st.sel[s];
                     const int sc = st.sel_cand[s];
-                    unsigned long long* T = d.tk[sel] + sc * tstride + st.tab_off[s];
-                    unsigned long long* V = d.tv + st.tab_off[s];
+                    unsigned long long* T = d.tk(sel) + sc * tstride + st.tab_off[s];
+                    unsigned long long* V = d.tv() + st.tab_off[s];
                     const int cap = st.cap_log2[s];
                     unsigned first = 0;
                     int bad = 0;
                     auto global_min = [&](unsigned long long key, long long slot, bool fr, unsigned long long packed) {
                         if (fr) {
                             const int k = atomicAdd(&st.dcnt[sel][li][sc], 1);
-                            d.dirty[sel][sc * dstride + a + k] =
+                            d.dirty(sel)[sc * dstride + a + k] =
                                 static_cast<uint32_t>(sc * tstride + st.tab_off[s] + slot);
                         }
                         if (atomicMin(V + slot, packed) == kEmptyVal) {
@@ -1374,6 +1832,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                         }
                     };
                     const int lane = tid & 31;
+#pragma unroll 1
                     for (int base = a + (tid - lane); base < b; base += kInFlight * kThreads) {  // warp-uniform
                         float4 q4[kInFlight];
 #pragma unroll
@@ -1427,6 +1886,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     int ng = nl;
                     if (owning) {
                         unsigned short* glist = list + kSelSlots;
+#pragma unroll 1
                         for (int k0 = tid - lane; k0 < nl; k0 += kThreads) {  // warp-uniform
                             const int k = k0 + lane;
                             const int si = (k < nl) ? static_cast<int>(list[k]) : 0;
@@ -1449,6 +1909,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                         gl = glist;
                         ng = static_cast<int>(st.gl_n);
                     }
+#pragma unroll 1
                     for (int k0 = tid - lane; k0 < ng; k0 += kProbes * kThreads) {  // warp-uniform
                         unsigned long long key[kProbes];
                         unsigned long long* Tp[kProbes];
@@ -1471,13 +1932,14 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                             // logged, warp-aggregated
                             const int pos = warp_append(ok && fr[u], &st.dcnt[sel][li][sc]);
                             if (pos >= 0)
-                                d.dirty[sel][sc * dstride + a + pos] =
+                                d.dirty(sel)[sc * dstride + a + pos] =
                                     static_cast<uint32_t>(sc * tstride + st.tab_off[s] + slot[u]);
                             if (ok) global_min(key[u], slot[u], false, sval[sidx[u]]);
                         }
                     }
                     if (bad) seg_error(d, s, bad);
                     const unsigned total = block_sum(first, st.scan_u);  // (its barriers order bh)
+#pragma unroll 1
                     for (int k = tid; k < kHistBins; k += kThreads)
                         if (st.bh[k]) atomicAdd(&hist[static_cast<long long>(s) * kHistBins + k], st.bh[k]);
                     if (tid == 0) st.ocnt[li] = owning ? static_cast<int>(st.rest_n) : 0;
@@ -1490,7 +1952,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             if (tid < S) {
                 st.kstar[tid] = static_cast<int>(ld_volatile(reinterpret_cast<const int*>(&ls[tid].kstar)));
                 if (blockIdx.x == 0) {
-                    hav_layer_trace* tr = d.tr + (static_cast<long long>(j) * S + tid) * kMaxLayers + l;
+                    hav_layer_trace* tr = d.tr() + (static_cast<long long>(j) * S + tid) * kMaxLayers + l;
                     tr->k_star = st.kstar[tid];
                     tr->accepted = (st.flags[tid] & F_ACCEPT) ? 1 : 0;
                     tr->s_star = (st.flags[tid] & F_ACTIVE) ? st.s_star[tid] : 0.0f;
@@ -1500,6 +1962,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             __syncthreads();
             {
                 int li = 0;
+#pragma unroll 1
                 for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
                     int a, b;
                     const int s = item_range(st, S, it, &a, &b);
@@ -1538,27 +2001,28 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     const int sel = st.sel[s];
                     const int sc = st.sel_cand[s];
                     const int c = st.dcnt[sel][li][sc];
-                    const uint32_t* lg = d.dirty[sel] + sc * dstride + a;
+                    const uint32_t* lg = d.dirty(sel) + sc * dstride + a;
                     const long long voff = sc * tstride;
                     const long long C = 1ll << st.cap_log2[s];
                     const int bin = st.cut_bin;
+#pragma unroll 1
                     for (int k = tid; k < c; k += kThreads) {
                         const uint32_t gs = lg[k];
-                        const unsigned long long v = d.tv[gs - voff];
+                        const unsigned long long v = d.tv()[gs - voff];
                         if (v == kEmptyVal) continue;
                         const int g = static_cast<int>(v & 0xffffffffull);
                         if (!cut) {
-                            mark_taken(taken, ord, d.posof, g);
+                            mark_taken(taken, ord, d.posof(), g);
                             continue;
                         }
-                        const unsigned long long h = priority(d.tk[sel][gs]);
+                        const unsigned long long h = priority(d.tk(sel)[gs]);
                         const int hb = static_cast<int>(h >> (64 - kHistBits));
                         if (hb < bin) {
-                            mark_taken(taken, ord, d.posof, g);
+                            mark_taken(taken, ord, d.posof(), g);
                         } else if (hb == bin) {
                             const uint32_t ci = atomicAdd(&ls[s].cand, 1u);
                             if (static_cast<long long>(ci) < (C >> 1)) {
-                                Cand* cd = d.cand + st.cand_off[s] + ci;
+                                Cand* cd = d.cand() + st.cand_off[s] + ci;
                                 cd->h = h;
                                 cd->g = static_cast<uint32_t>(g);
                             } else {
@@ -1568,17 +2032,18 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     }
                     // the voxels the selection kept out of the table (owned whole)
                     const int oc = st.ocnt[li];
-                    const Cand* ol = reinterpret_cast<const Cand*>(d.ord[(j + 1) & 1]) + a;
+                    const Cand* ol = reinterpret_cast<const Cand*>(d.ord((j + 1) & 1)) + a;
+#pragma unroll 1
                     for (int k = tid; k < oc; k += kThreads) {
                         const unsigned long long h = ol[k].h;
                         const int g = static_cast<int>(ol[k].g);
                         const int hb = static_cast<int>(h >> (64 - kHistBits));
                         if (!cut || hb < bin) {
-                            mark_taken(taken, ord, d.posof, g);
+                            mark_taken(taken, ord, d.posof(), g);
                         } else if (hb == bin) {
                             const uint32_t ci = atomicAdd(&ls[s].cand, 1u);
                             if (static_cast<long long>(ci) < (C >> 1)) {
-                                Cand* cd = d.cand + st.cand_off[s] + ci;
+                                Cand* cd = d.cand() + st.cand_off[s] + ci;
                                 cd->h = h;
                                 cd->g = static_cast<uint32_t>(g);
                             } else {
@@ -1605,16 +2070,18 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 if (tid < S) st.cprefix[tid] = cpre;
                 if (tid == 0) st.cprefix[S] = ctot;
                 __syncthreads();
+#pragma unroll 1
                 for (long long w = gtid; w < ctot; w += gstride) {
                     const int s = find_seg(st.cprefix, S, w);
                     const int jdx = static_cast<int>(w) - st.cprefix[s];
                     const int cs = st.cprefix[s + 1] - st.cprefix[s];
-                    const Cand* base = d.cand + st.cand_off[s];
+                    const Cand* base = d.cand() + st.cand_off[s];
                     const unsigned long long hj = base[jdx].h;
                     int rank = 0;
+#pragma unroll 1
                     for (int k = 0; k < cs; ++k) rank += (base[k].h < hj) ? 1 : 0;
                     const int r = st.ml[s] - static_cast<int>(ls[s].below);
-                    if (rank < r) mark_taken(taken, ord, d.posof, static_cast<int>(base[jdx].g));
+                    if (rank < r) mark_taken(taken, ord, d.posof(), static_cast<int>(base[jdx].g));
                 }
                 int sf = 0;
                 if (tid < S && (st.flags[tid] & F_ACTIVE) && st.kstar[tid] < st.ml[tid]) sf = 1;
@@ -1623,66 +2090,76 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 if (sf) st.any = 1;
                 __syncthreads();
                 if (st.any) {
+#pragma unroll 1
                     for (int s = 0; s < S; ++s) {
                         if (!((st.flags[s] & F_ACTIVE) && st.kstar[s] < st.ml[s])) continue;
                         const int n = st.n[s];
                         const int a = static_cast<int>(st.off[s] + static_cast<long long>(n) * blockIdx.x / nb);
                         const int b = static_cast<int>(st.off[s] + static_cast<long long>(n) * (blockIdx.x + 1) / nb);
                         int cnt = 0;
+#pragma unroll 1
                         for (int g = a + tid; g < b; g += kThreads) cnt += is_taken(taken, g) ? 0 : 1;
                         int tot;
                         block_excl_scan<int>(cnt, &tot, st.scan_i);
-                        if (tid == 0) d.psf[static_cast<long long>(s) * kMaxBlocks + blockIdx.x] = tot;
+                        if (tid == 0) d.psf()[static_cast<long long>(s) * kMaxBlocks + blockIdx.x] = tot;
                     }
                 }
                 // every candidate table of every set, and the value table, back to
                 // empty, slot by slot
                 int li = 0;
+#pragma unroll 1
                 for (int it = blockIdx.x; it < st.items_total; it += nb, ++li) {
                     int a, b;
                     const int s = item_range(st, S, it, &a, &b);
                     const bool act = (st.flags[s] & F_ACTIVE) != 0;
+#pragma unroll 1
                     for (int t = 0; t < kTableSets; ++t) {
+#pragma unroll 1
                         for (int cd = 0; cd < ncand; ++cd) {
                             const int c2 = st.dcnt[t][li][cd];
                             const bool v_too = act && st.sel[s] == t && st.sel_cand[s] == cd;
-                            const uint32_t* lg = d.dirty[t] + cd * dstride + a;
+                            const uint32_t* lg = d.dirty(t) + cd * dstride + a;
                             const long long voff = cd * tstride;
+#pragma unroll 4
                             for (int k = tid; k < c2; k += kThreads) {
                                 const uint32_t gs = lg[k];
-                                d.tk[t][gs] = kEmptyKey;
-                                if (v_too) d.tv[gs - voff] = kEmptyVal;
+                                d.tk(t)[gs] = kEmptyKey;
+                                if (v_too) d.tv()[gs - voff] = kEmptyVal;
                             }
                         }
                     }
                 }
                 __syncthreads();
+#pragma unroll 1
                 for (int k = tid; k < kTableSets * kLocalItems * kMaxCand; k += kThreads)
                     (&st.dcnt[0][0][0])[k] = 0;
                 if (l + 1 < P.layers) clear_layer_state(d, S, q ^ 1, gtid, gstride);
                 if (!grid_sync(d, nb, st, TAG(5, j, l, 0))) return;
                 if (j + 1 == P.L && l + 1 == P.layers && blockIdx.x == 0 && tid == 0)
-                    *(volatile unsigned*)d.clean = 1u;  // every table slot is empty again
+                    *(volatile unsigned*)d.clean() = 1u;  // every table slot is empty again
             }
             // ------------------------------------------------ shortfall fill
             if (st.any) {
+#pragma unroll 1
                 for (int s = 0; s < S; ++s) {
                     if (!((st.flags[s] & F_ACTIVE) && st.kstar[s] < st.ml[s])) continue;
                     int pre = 0;
+#pragma unroll 1
                     for (int b = tid; b < static_cast<int>(blockIdx.x); b += kThreads)
-                        pre += d.psf[static_cast<long long>(s) * kMaxBlocks + b];
+                        pre += d.psf()[static_cast<long long>(s) * kMaxBlocks + b];
                     int tot;
                     block_excl_scan<int>(pre, &tot, st.scan_i);
                     int budget = (st.ml[s] - st.kstar[s]) - tot;
                     const int n = st.n[s];
                     const int a = static_cast<int>(st.off[s] + static_cast<long long>(n) * blockIdx.x / nb);
                     const int b = static_cast<int>(st.off[s] + static_cast<long long>(n) * (blockIdx.x + 1) / nb);
+#pragma unroll 1
                     for (int g0 = a; g0 < b && budget > 0; g0 += kThreads) {
                         const int g = g0 + tid;
                         const int free_pt = (g < b && !is_taken(taken, g)) ? 1 : 0;
                         int chunk;
                         const int rank = block_excl_scan<int>(free_pt, &chunk, st.scan_i);
-                        if (free_pt && rank < budget) mark_taken(taken, ord, d.posof, g);
+                        if (free_pt && rank < budget) mark_taken(taken, ord, d.posof(), g);
                         budget -= chunk;
                     }
                 }
@@ -1693,7 +2170,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
         // ---------------------------------------------------- compaction
         // Segments in error take their first m points, so every other
         // segment's output positions stay exact.
-        if (tid < S) st.err[tid] = ld_volatile(&d.sh[tid].status);
+        if (tid < S) st.err[tid] = ld_volatile(&d.sh()[tid].status);
         if (tid == 0) st.any = 0;
         __syncthreads();
         if (tid < S && st.err[tid]) st.any = 1;
@@ -1708,6 +2185,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             const long long g0 = w * 32;
             if (g0 + 32 > NL) bits &= (NL - g0 >= 32) ? 0xffffffffu : ((1u << (NL - g0)) - 1u);
             if (any_err) {
+#pragma unroll 1
                 for (int k = 0; k < 32 && g0 + k < NL; ++k) {
                     const int s = find_seg(st.off, S, g0 + k);
                     if (st.err[s]) {
@@ -1725,42 +2203,45 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
         {
             // level j+1 accumulates its bounding box in the parity level j-1 used
             if (blockIdx.x == 0 && tid < S)
-                for (int a = 0; a < 6; ++a) d.sh[tid].bbox[(j + 1) & 1][a] = 0u;
+                for (int a = 0; a < 6; ++a) d.sh()[tid].bbox[(j + 1) & 1][a] = 0u;
             // ascending order: per-word block-local prefixes and the block total
             unsigned run = 0;
+#pragma unroll 1
             for (long long w0 = wb; w0 < we; w0 += kThreads) {
                 const long long w = w0 + tid;
                 const unsigned c = (w < we) ? __popc(eff_word(w)) : 0u;
                 unsigned tot;
                 const unsigned before = block_excl_scan<unsigned>(c, &tot, st.scan_u);
-                if (w < we) d.wpre[w] = run + before;
+                if (w < we) d.wpre()[w] = run + before;
                 run += tot;
             }
-            if (tid == 0) d.pcmp[blockIdx.x] = static_cast<int32_t>(run);
+            if (tid == 0) d.pcmp()[blockIdx.x] = static_cast<int32_t>(run);
             // processing order: kept points per owned item
             if (!last_level) {
+#pragma unroll 1
                 for (int it = blockIdx.x; it < st.items_total; it += nb) {
                     int a, b;
                     const int s = item_range(st, S, it, &a, &b);
                     unsigned c = 0;
+#pragma unroll 4
                     for (int i = a + tid; i < b; i += kThreads)
                         c += eff_taken(s, level_index(ord[i].w)) ? 1u : 0u;
                     const unsigned tot = block_sum(c, st.scan_u);
-                    if (tid == 0) d.pitem[it] = static_cast<int32_t>(tot);
+                    if (tid == 0) d.pitem()[it] = static_cast<int32_t>(tot);
                 }
             }
             if (!grid_sync(d, nb, st, TAG(7, j, 0, 0))) return;
         }
         {
             // prefixes of every block's count and (next level) every item's count
-            if (tid == 0) st.set_clean = 0;
             int* pre_blk = reinterpret_cast<int*>(dyn);
             int* pre_item = pre_blk + kMaxBlocks;
             {
                 int run = 0;
+#pragma unroll 1
                 for (int b0 = 0; b0 < static_cast<int>(nb); b0 += kThreads) {
                     const int b = b0 + tid;
-                    const int c = (b < static_cast<int>(nb)) ? d.pcmp[b] : 0;
+                    const int c = (b < static_cast<int>(nb)) ? d.pcmp()[b] : 0;
                     int tot;
                     const int before = block_excl_scan<int>(c, &tot, st.scan_i);
                     if (b < static_cast<int>(nb)) pre_blk[b] = run + before;
@@ -1768,9 +2249,10 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 }
                 if (!last_level) {
                     run = 0;
+#pragma unroll 1
                     for (int i0 = 0; i0 < st.items_total; i0 += kThreads) {
                         const int it = i0 + tid;
-                        const int c = (it < st.items_total) ? d.pitem[it] : 0;
+                        const int c = (it < st.items_total) ? d.pitem()[it] : 0;
                         int tot;
                         const int before = block_excl_scan<int>(c, &tot, st.scan_i);
                         if (it < st.items_total) pre_item[it] = run + before;
@@ -1786,19 +2268,20 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 while (b + 1 < static_cast<long long>(nb) && W * (b + 1) / nb <= w) ++b;
                 while (b > 0 && W * b / nb > w) --b;
                 const uint32_t below = eff_word(w) & ((1u << (g & 31)) - 1u);
-                return static_cast<long long>(pre_blk[b]) + d.wpre[w] + __popc(below);
+                return static_cast<long long>(pre_blk[b]) + d.wpre()[w] + __popc(below);
             };
             int32_t* out = P.out[j];
-            int32_t* orig_out = d.orig[j & 1];
+            int32_t* orig_out = d.orig(j & 1);
+#pragma unroll 1
             for (long long w = wb + tid; w < we; w += kThreads) {
                 uint32_t bits = eff_word(w);
-                long long pos = static_cast<long long>(pre_blk[blockIdx.x]) + d.wpre[w];
+                long long pos = static_cast<long long>(pre_blk[blockIdx.x]) + d.wpre()[w];
                 while (bits) {
                     const int k = __ffs(bits) - 1;
                     bits &= bits - 1;
                     const long long g = w * 32 + k;
                     if (pos >= st.m_total) {  // cannot happen: every segment takes exactly m
-                        atomicCAS(&d.gh->status, 0, static_cast<int>(HAV_ERR_TABLE_FULL));
+                        atomicCAS(&d.gh()->status, 0, static_cast<int>(HAV_ERR_TABLE_FULL));
                         break;
                     }
                     const int s = find_seg(st.off, S, g);
@@ -1809,42 +2292,69 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 }
             }
             if (!last_level) {
-                float4* ord_out = d.ord[(j + 1) & 1];
+                float4* ord_out = d.ord((j + 1) & 1);
                 const int npar = (j + 1) & 1;
+#pragma unroll 1
                 for (int it = blockIdx.x; it < st.items_total; it += nb) {
                     int a, b;
                     const int s = item_range(st, S, it, &a, &b);
                     long long base = pre_item[it];
                     // the next level's bounding box over the points kept here
                     float mnv[3] = {INFINITY, INFINITY, INFINITY}, mxv[3] = {-INFINITY, -INFINITY, -INFINITY};
-                    for (int i0 = a; i0 < b; i0 += kThreads) {
-                        const int i = i0 + tid;
-                        float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                        int keep = 0;
-                        if (i < b) {
-                            q4 = ord[i];
-                            keep = eff_taken(s, level_index(q4.w)) ? 1 : 0;
+                    // four points a thread per step: the kept ones ranked by warp ballots
+                    // and one prefix over the (round, warp) counts
+                    constexpr int kW = kThreads / 32;
+                    static_assert(4 * kW <= 64, "two counts a lane");
+                    const int lane = tid & 31, wid = tid >> 5;
+#pragma unroll 1
+                    for (int i0 = a; i0 < b; i0 += 4 * kThreads) {
+                        float4 q4[4];
+                        unsigned m[4];
+                        bool keep[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) q4[k] = ord[min(i0 + k * kThreads + tid, b - 1)];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            keep[k] = i0 + k * kThreads + tid < b && eff_taken(s, level_index(q4[k].w));
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            m[k] = __ballot_sync(0xffffffffu, keep[k]);
+                            if (lane == 0) st.gcnt[k * kW + wid] = __popc(m[k]);
                         }
-                        int tot;
-                        const int rank = block_excl_scan<int>(keep, &tot, st.scan_i);
-                        if (keep) {
-                            const long long pos2 = base + rank;
-                            const long long ng = pos_asc(level_index(q4.w));
-                            if (pos2 < st.m_total && ng < st.m_total) {
-                                ord_out[pos2] = make_float4(q4.x, q4.y, q4.z, __int_as_float(static_cast<int>(ng)));
-                                d.posof[ng] = static_cast<int32_t>(pos2);
+                        __syncthreads();
+                        if (wid == 0) {
+                            const int c0 = 2 * lane < 4 * kW ? st.gcnt[2 * lane] : 0;
+                            const int c1 = 2 * lane < 4 * kW ? st.gcnt[2 * lane + 1] : 0;
+                            const int e = warp_incl_scan(c0 + c1);
+                            if (2 * lane < 4 * kW) {
+                                st.gcnt[2 * lane] = e - c0 - c1;
+                                st.gcnt[2 * lane + 1] = e - c1;
                             }
-                            mnv[0] = fminf(mnv[0], q4.x);
-                            mnv[1] = fminf(mnv[1], q4.y);
-                            mnv[2] = fminf(mnv[2], q4.z);
-                            mxv[0] = fmaxf(mxv[0], q4.x);
-                            mxv[1] = fmaxf(mxv[1], q4.y);
-                            mxv[2] = fmaxf(mxv[2], q4.z);
+                            if (lane == 31) st.gcnt[64] = e;
                         }
-                        base += tot;
+                        __syncthreads();
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (!keep[k]) continue;
+                            const long long pos2 = base + st.gcnt[k * kW + wid] + __popc(m[k] & ((1u << lane) - 1u));
+                            const long long ng = pos_asc(level_index(q4[k].w));
+                            if (pos2 < st.m_total && ng < st.m_total) {
+                                ord_out[pos2] = make_float4(q4[k].x, q4[k].y, q4[k].z, __int_as_float(static_cast<int>(ng)));
+                                d.posof()[ng] = static_cast<int32_t>(pos2);
+                            }
+                            mnv[0] = fminf(mnv[0], q4[k].x);
+                            mnv[1] = fminf(mnv[1], q4[k].y);
+                            mnv[2] = fminf(mnv[2], q4[k].z);
+                            mxv[0] = fmaxf(mxv[0], q4[k].x);
+                            mxv[1] = fmaxf(mxv[1], q4[k].y);
+                            mxv[2] = fmaxf(mxv[2], q4[k].z);
+                        }
+                        base += st.gcnt[64];
+                        __syncthreads();
                     }
 #pragma unroll
                     for (int a3 = 0; a3 < 3; ++a3) {
+#pragma unroll 1
                         for (int o = 16; o > 0; o >>= 1) {
                             mnv[a3] = fminf(mnv[a3], __shfl_xor_sync(0xffffffffu, mnv[a3], o));
                             mxv[a3] = fmaxf(mxv[a3], __shfl_xor_sync(0xffffffffu, mxv[a3], o));
@@ -1859,18 +2369,19 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                     __syncthreads();
                     if (tid < 6) {
                         float r = st.redf[tid][0];
+#pragma unroll 1
                         for (int w = 1; w < kThreads / 32; ++w)
                             r = (tid < 3) ? fminf(r, st.redf[tid][w]) : fmaxf(r, st.redf[tid][w]);
                         if (isfinite(r)) {
-                            if (tid < 3) atomicMax(&d.sh[s].bbox[npar][tid], ~enc_f(r));
-                            else atomicMax(&d.sh[s].bbox[npar][tid], enc_f(r));
+                            if (tid < 3) atomicMax(&d.sh()[s].bbox[npar][tid], ~enc_f(r));
+                            else atomicMax(&d.sh()[s].bbox[npar][tid], enc_f(r));
                         }
                     }
                     __syncthreads();
                 }
                 // the next level's taken mask, layer states and search prefix
-                fill<uint32_t>(d.taken[npar], st.m_total / 32 + 1, 0u, gtid, gstride);
-                fill<int32_t>(d.prefix, static_cast<long long>(S) * kMaxIters, -1, gtid, gstride);
+                fill<uint32_t>(d.taken(npar), st.m_total / 32 + 1, 0u, gtid, gstride);
+                fill<int32_t>(d.prefix(), static_cast<long long>(S) * kMaxIters, -1, gtid, gstride);
                 clear_layer_state(d, S, 0, gtid, gstride);
                 clear_layer_state(d, S, 1, gtid, gstride);
                 if (!grid_sync(d, nb, st, TAG(8, j, 0, 0))) return;

@@ -56,6 +56,7 @@ constexpr int kSelMax = 8192;    // slots of a CTA's part of the selection table
 constexpr int kMaxQ = 16;        // largest cluster
 constexpr int kCutBits = 6;      // cut-off histogram over the top priority bits
 constexpr int kCutBins = 1 << kCutBits;
+constexpr int kMaxOpen = 128;    // undecided points of a pass that are compared with one another
 constexpr int kCandAll = 1024;   // boundary-bin candidates of the cluster that every CTA receives
 constexpr size_t kPtsBytes = static_cast<size_t>(kPtsSmem) * 16;
 constexpr size_t kTabBytes = static_cast<size_t>(kSelMax) * 16;
@@ -129,6 +130,7 @@ struct SmallSmem {
     uint32_t own_hist[kCutBins];
     int bin_cnt[kMaxQ];  // records of this CTA's share by owner: counts, then places
     unsigned nlist;           // slots the selection filled
+    int nopen[2];             // undecided points of a kHash round, by its parity
     unsigned own_cand;        // this CTA's boundary-bin candidates, at the front of the slot list
     int cut_bin, cut_below, kstar;
     unsigned eb;
@@ -293,6 +295,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
     const bool hash = pg->mode == kHash;
     const unsigned nslots = pg->nslots;
     unsigned mult = 0x9E3779B1u;
+    if (threadIdx.x == 0) smem().nopen[0] = 0;
     {
         const CellMap cell(pg->bg);
 #pragma unroll 1
@@ -335,7 +338,8 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
         }
         return won;
     }
-    unsigned long long open = ~0ull;  // bit k: point tid + k kST is undecided
+    unsigned long long open = ~0ull;  // bit k: point t0 + k T is undecided
+    unsigned short* const open_list = reinterpret_cast<unsigned short*>(dyn + kListOff);
 #pragma unroll 1
     for (int round = 0; round < n; ++round) {  // (every round decides a cell at least)
         unsigned long long left = 0;
@@ -356,8 +360,28 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
                     else if (area[w[k]] != c[k]) left |= 1ull << (k0 + k);
                 }
         }
+        // a few undecided points are settled among themselves (one counts where no
+        // earlier one has its cell), many take another round
+        SmallSmem& sm = smem();
+        if (left) {
+            int pos = atomicAdd(&sm.nopen[round & 1], __popcll(left));
+            for (unsigned long long b = left; b; b &= b - 1ull, ++pos)
+                if (pos < kST) open_list[pos] = static_cast<unsigned short>(t0 + (__ffsll(static_cast<long long>(b)) - 1) * T);
+        }
+        __syncthreads();
+        const int c = sm.nopen[round & 1];
+        if (threadIdx.x == 0) sm.nopen[(round + 1) & 1] = 0;
+        if (c <= kMaxOpen) {
+            if (static_cast<int>(threadIdx.x) < c) {
+                const unsigned mine = area[open_list[threadIdx.x]];
+                bool seen = false;
+                for (int k = 0; k < static_cast<int>(threadIdx.x) && !seen; ++k) seen = area[open_list[k]] == mine;
+                won += seen ? 0u : 1u;
+            }
+            break;
+        }
+        __syncthreads();
         open = left;
-        if (!__syncthreads_or(left != 0ull)) break;
         mult = mult * 0x85EBCA77u + 0xC2B2AE3Eu;  // (odd again)
         for (; left; left &= left - 1ull) {
             const int i = t0 + (__ffsll(static_cast<long long>(left)) - 1) * T;
