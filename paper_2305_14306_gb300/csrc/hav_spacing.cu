@@ -10,8 +10,15 @@
 // split over a second grid dimension so that small subsets still fill the
 // GPU; the partial minima meet in an atomicMin on the float bits (squared
 // distances are non-negative, so their bit patterns order like the values).
+// Bound by the nine binary32 operations of a pair; ranges of 32 candidates and
+// more (1,024 before) leave no SM idle below 32,768 points.  With its histogram
+// on GB300: 1,000 points 38 us (92), 8,192 points 40 us (96), 16,384 points 105
+// us (146), 32,000 points 318 us (509); from kSpacingGridMin on, the search on
+// a grid takes over.
 
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "hav.h"
 #include "hav_device.cuh"
@@ -23,6 +30,7 @@ namespace {
 constexpr int kSpThreads = 256;
 constexpr int kSpQ = 4;        // query points per thread
 constexpr int kSpTile = 1024;  // candidates per shared-memory tile
+constexpr int kSpRange = 32;   // candidate ranges are multiples of this
 constexpr unsigned kInfBits = 0x7f800000u;
 
 __global__ void spacing_init(unsigned* out, long long m) {
@@ -61,28 +69,35 @@ __global__ void __launch_bounds__(kSpThreads) spacing_kernel(const float* pts, l
     const long long c1 = (c0 + chunk < m) ? c0 + chunk : m;
     for (long long t0 = c0; t0 < c1; t0 += kSpTile) {
         __syncthreads();
-        for (int k = tid; k < kSpTile; k += kSpThreads) {
+        const int cnt = static_cast<int>((c1 - t0 < kSpTile) ? c1 - t0 : kSpTile);
+        for (int k = tid; k < cnt; k += kSpThreads) {
             const long long j = t0 + k;
-            float4 b = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(-1));  // w: subset position, -1 = none
+            float4 b = make_float4(NAN, NAN, NAN, 0.0f);  // none: no distance to it is below another
             if (j < c1) {
                 const int32_t i = idx[j];
-                if (i >= 0 && i < n)
-                    b = make_float4(pts[3ll * i], pts[3ll * i + 1], pts[3ll * i + 2], __int_as_float(static_cast<int>(j)));
+                if (i >= 0 && i < n) b = make_float4(pts[3ll * i], pts[3ll * i + 1], pts[3ll * i + 2], 0.0f);
             }
             tile[k] = b;
         }
         __syncthreads();
-        const int cnt = static_cast<int>((c1 - t0 < kSpTile) ? c1 - t0 : kSpTile);
-        for (int k = 0; k < cnt; ++k) {
-            const float4 b = tile[k];
-            const int j = __float_as_int(b.w);
+        // (fminf passes a NaN by; only a tile that overlaps the block's own points
+        // needs the test against the point itself)
+        auto pairs = [&](auto own) {
+#pragma unroll 4
+            for (int k = 0; k < cnt; ++k) {
+                const float4 b = tile[k];
 #pragma unroll
-            for (int u = 0; u < kSpQ; ++u) {
-                const float dx = __fsub_rn(qx[u], b.x), dy = __fsub_rn(qy[u], b.y), dz = __fsub_rn(qz[u], b.z);
-                const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-                if (j >= 0 && j != qpos[u] && d2 < best[u]) best[u] = d2;
+                for (int u = 0; u < kSpQ; ++u) {
+                    const float dx = __fsub_rn(qx[u], b.x), dy = __fsub_rn(qy[u], b.y), dz = __fsub_rn(qz[u], b.z);
+                    const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+                    if (!own.value || t0 + k != qpos[u]) best[u] = fminf(best[u], d2);
+                }
             }
-        }
+        };
+        if (t0 < qbase + kSpThreads * kSpQ && qbase < t0 + cnt)
+            pairs(std::true_type{});
+        else
+            pairs(std::false_type{});
     }
 #pragma unroll
     for (int u = 0; u < kSpQ; ++u)
@@ -142,12 +157,12 @@ int launch_spacing(const float* points, long long n, const int32_t* idx, long lo
                    int32_t* status, int sms, cudaStream_t stream) {
     unsigned* out = reinterpret_cast<unsigned*>(out_d2);
     const long long qblocks = (m + kSpThreads * kSpQ - 1) / (kSpThreads * kSpQ);
-    long long tiles = (m + kSpTile - 1) / kSpTile;
+    long long tiles = (m + kSpRange - 1) / kSpRange;
     long long want = (4ll * sms + qblocks - 1) / qblocks;  // candidate ranges per query block
     if (want > tiles) want = tiles;
     if (want > 65535) want = 65535;
     if (want < 1) want = 1;
-    const long long chunk = ((tiles + want - 1) / want) * kSpTile;
+    const long long chunk = ((tiles + want - 1) / want) * kSpRange;
     const long long splits = (m + chunk - 1) / chunk;
     long long ib = (m + 255) / 256;
     int launched = 1;
