@@ -177,16 +177,17 @@ constexpr int kMagicBits = 0x4B400000;
 // fast grid; false where an axis is near an integer (one point in 10^4 to 10^5
 // of a scene).  Without conversion or rounding instructions, which run at a
 // fraction of the rate of additions: k = (q + kMagic) - kMagic, and the bits of
-// q + kMagic are kMagicBits + k.  (|q| >= 2^22: |k| amb exceeds v / 2, so the
+// q + kMagic are kMagicBits + k; six instructions an axis.  (|q| >= 2^22: |k| amb exceeds v / 2, so the
 // near case takes it.)
 __device__ __forceinline__ bool floor_bits(const float p[3], const float r[3], const float v[3], float amb, int t[3]) {
+    const float amb0 = __fmul_rn(amb, 8.4703294725430034e-22f);  // 2^-70 amb
     bool ok = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float s = __fadd_rn(__fmul_rn(p[a], r[a]), kMagic);
+        const float s = __fmaf_rn(p[a], r[a], kMagic);
         const float k = __fsub_rn(s, kMagic);
         const float rem = __fmaf_rn(-k, v[a], p[a]);
-        ok = ok && fabsf(rem) > __fmul_rn(__fadd_rn(fabsf(k), 8.4703294725430034e-22f), amb);  // (|k| + 2^-70) amb
+        ok = ok && fabsf(rem) > __fmaf_rn(fabsf(k), amb, amb0);
         t[a] = __float_as_int(s) + (__float_as_int(rem) >> 31);
     }
     return ok;

@@ -16,14 +16,16 @@
 // distributed shared memory, and a pass of one step took 4.2-5.6 us (measured
 // on GB300, 16 CTAs, 16,384-20,876 points).  On one CTA the count costs no
 // atomics and nothing to empty, and a warp prepares the next grids meanwhile: a
-// pass over 1,000 points 2.3 -> 1.5 us.  What bounds both is latency: of a pass
-// of 1,000 points, 1.3 us are short serial sections of a few dozen
-// instructions between barriers; of one of 16,384 points on a cluster, half
-// are the points (11 cycles a point and SM) and half such sections.  Measured
-// on GB300, whole calls: 1,000-point room to 250 57.5 -> 43.0 us, 16,384
-// uniform points to 4,096 80.4 -> 69.3 us, LiDAR chain 20,876 -> 16,384 ->
-// 4,096 -> 1,024 -> 512 347 -> 329 us, 64 clouds of 1,000-4,000 points, two
-// levels, 141 -> 103 us.
+// pass over 1,000 points 2.3 -> 1.5 us.  What bounds both is latency and the
+// instructions of a point: of a pass of 1,000 points, 1.3 us are short serial
+// sections of a few dozen instructions between barriers; of one of 20,876
+// points on 16 CTAs, 13 us in the finest sizes of a LiDAR scan, 6 us are the
+// points' cells (each CTA sees all of them: 36 instructions a point), 4 the
+// look at the words (a third of it their random bank conflicts), 1.5 the
+// undecided points and the rest such sections.  Measured on GB300, whole calls:
+// 1,000-point room to 250 57.5 -> 43.7 us, 16,384 uniform points to 4,096 80.4
+// -> 63.6 us, LiDAR chain 20,876 -> 16,384 -> 4,096 -> 1,024 -> 512 364 -> 289
+// us, 64 clouds of 1,000-4,000 points, two levels, 144 -> 105 us.
 //
 // The selection at s* is spread by voxel: every CTA goes through all points
 // and keeps those whose voxel hashes to it, so that the table of a voxel's
@@ -35,6 +37,8 @@
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "hav.h"
 #include "hav_device.cuh"
@@ -56,7 +60,9 @@ constexpr int kSelMax = 8192;    // slots of a CTA's part of the selection table
 constexpr int kMaxQ = 16;        // largest cluster
 constexpr int kCutBits = 6;      // cut-off histogram over the top priority bits
 constexpr int kCutBins = 1 << kCutBits;
-constexpr int kMaxOpen = 128;    // undecided points of a pass that are compared with one another
+constexpr int kOpenA = kSelMax / 4 * 3;  // undecided points of a pass that are listed (in later rounds, alternately the rest)
+constexpr unsigned kManyOpen = 0xffffffffu;
+constexpr int kMaxOpen = 32;     // undecided points of a pass that a warp compares with one another
 constexpr int kCandAll = 1024;   // boundary-bin candidates of the cluster that every CTA receives
 constexpr size_t kPtsBytes = static_cast<size_t>(kPtsSmem) * 16;
 constexpr size_t kTabBytes = static_cast<size_t>(kSelMax) * 16;
@@ -285,25 +291,38 @@ __device__ __forceinline__ uint32_t* pass_area() {
 
 // kDirect and kHash: the cells this thread's points (t0, t0 + T, ...) stand for.  The area holds
 // the points' cell numbers and nslots 16-bit words behind them.
-template <bool SM>
-__device__ __noinline__ unsigned count_cells(const float4* stg, int n, const PassGrid* pg, int t0, int T) {
-    // points a thread loads ahead: global loads need more of them in flight
-    constexpr int kIn = SM ? 4 : 8;
+template <bool SM, int T>
+__device__ __noinline__ unsigned count_cells(const float4* stg, int n, const PassGrid* pg, int t0) {
+    // Points of a group: more of them cost padding in the last group and code (16 / 8 /
+    // 4 / 2 / 1 on 16 CTAs, LiDAR chain of 20,876 points: 343 / 291 / 275 / 288 / 320 us)
+    constexpr int kIn = (SM && T != kST) ? 2 : 4;
     static_assert(64 % kIn == 0 && kSmallMax <= 64 * kST, "one bit per point of a thread: n <= 64 T");
     uint32_t* const area = pass_area<SM>();
     unsigned short* const word = reinterpret_cast<unsigned short*>(area + n);
     const bool hash = pg->mode == kHash;
     const unsigned nslots = pg->nslots;
     unsigned mult = 0x9E3779B1u;
-    if (threadIdx.x == 0) smem().nopen[0] = 0;
+    SmallSmem& sm = smem();
+    if (threadIdx.x == 0) sm.nopen[0] = 0;
+    // group(i0, all): the points i0, i0 + T, ... of which `all`, or those below n, are there.
+    // A thread's loops run over whole groups, free of range checks, and one more
+    auto each = [&](auto&& group) {
+        int i0 = t0;
+        if constexpr (!SM) {
+#pragma unroll 1
+            for (; i0 + (kIn - 1) * T < n; i0 += kIn * T) group(i0, std::true_type{});
+        }
+#pragma unroll 1
+        for (; i0 < n; i0 += kIn * T) group(i0, std::false_type{});
+    };
     {
         const CellMap cell(pg->bg);
-#pragma unroll 1
-        for (int i0 = t0; i0 < n; i0 += kIn * T) {
+        each([&](int i0, auto all) {
             float4 q[kIn];
             unsigned c[kIn];
 #pragma unroll
-            for (int k = 0; k < kIn; ++k) q[k] = load_point<SM>(stg, min(i0 + k * T, n - 1));
+            for (int k = 0; k < kIn; ++k)
+                q[k] = load_point<SM>(stg, all.value ? i0 + k * T : min(i0 + k * T, n - 1));
             unsigned near = 0u;  // points near a cell's face: one branch for all of them
 #pragma unroll
             for (int k = 0; k < kIn; ++k) near |= cell.fast(q[k], &c[k]) ? 0u : (1u << k);
@@ -316,85 +335,148 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
             for (int k = 0; k < kIn; ++k) {
                 const int i = i0 + k * T;
                 if (__float_as_int(q[k].w) < 0) c[k] = kNoCell;  // taken
-                if (i < n) {
+                if (all.value || i < n) {
                     area[i] = c[k];
                     if (c[k] != kNoCell)
                         word[hash ? __umulhi(c[k] * mult, nslots) : c[k]] = static_cast<unsigned short>(i);
                 }
             }
-        }
+        });
     }
     __syncthreads();
     unsigned won = 0;
     if (!hash) {
-#pragma unroll 1
-        for (int i0 = t0; i0 < n; i0 += kIn * T) {
+        each([&](int i0, auto all) {
             unsigned c[kIn];
 #pragma unroll
-            for (int k = 0; k < kIn; ++k) c[k] = (i0 + k * T < n) ? area[i0 + k * T] : kNoCell;
+            for (int k = 0; k < kIn; ++k) c[k] = (all.value || i0 + k * T < n) ? area[i0 + k * T] : kNoCell;
 #pragma unroll
             for (int k = 0; k < kIn; ++k)
                 if (c[k] != kNoCell) won += (word[c[k]] == i0 + k * T) ? 1u : 0u;
-        }
+        });
         return won;
     }
-    unsigned long long open = ~0ull;  // bit k: point t0 + k T is undecided
-    unsigned short* const open_list = reinterpret_cast<unsigned short*>(dyn + kListOff);
-#pragma unroll 1
-    for (int round = 0; round < n; ++round) {  // (every round decides a cell at least)
-        unsigned long long left = 0;
-#pragma unroll 1
-        for (int k0 = 0, i0 = t0; i0 < n; k0 += kIn, i0 += kIn * T) {
-            const unsigned bits = static_cast<unsigned>(open >> k0) & ((1u << kIn) - 1u);
-            if (!bits) continue;
-            unsigned c[kIn], w[kIn];
+    // a slot's last writer stands for its cell; the points of the other cells that
+    // share the slot are listed (a bit per point, then their indices)
+    unsigned long long left = 0;
+    int k0 = 0;
+    each([&](int i0, auto all) {
+        unsigned c[kIn], w[kIn], bits = 0u;
 #pragma unroll
-            for (int k = 0; k < kIn; ++k)
-                c[k] = (((bits >> k) & 1u) && i0 + k * T < n) ? area[i0 + k * T] : kNoCell;
+        for (int k = 0; k < kIn; ++k) c[k] = (all.value || i0 + k * T < n) ? area[i0 + k * T] : kNoCell;
 #pragma unroll
-            for (int k = 0; k < kIn; ++k) w[k] = (c[k] != kNoCell) ? word[__umulhi(c[k] * mult, nslots)] : 0u;
+        for (int k = 0; k < kIn; ++k) w[k] = (c[k] != kNoCell) ? word[__umulhi(c[k] * mult, nslots)] : 0u;
 #pragma unroll
-            for (int k = 0; k < kIn; ++k)
-                if (c[k] != kNoCell) {
-                    if (w[k] == static_cast<unsigned>(i0 + k * T)) ++won;
-                    else if (area[w[k]] != c[k]) left |= 1ull << (k0 + k);
-                }
+        for (int k = 0; k < kIn; ++k) {
+            const unsigned other = area[w[k]];
+            if (c[k] != kNoCell) {
+                won += (w[k] == static_cast<unsigned>(i0 + k * T)) ? 1u : 0u;
+                bits |= (other != c[k]) ? (1u << k) : 0u;
+            }
         }
-        // a few undecided points are settled among themselves (one counts where no
-        // earlier one has its cell), many take another round
-        SmallSmem& sm = smem();
-        if (left) {
-            int pos = atomicAdd(&sm.nopen[round & 1], __popcll(left));
-            for (unsigned long long b = left; b; b &= b - 1ull, ++pos)
-                if (pos < kST) open_list[pos] = static_cast<unsigned short>(t0 + (__ffsll(static_cast<long long>(b)) - 1) * T);
+        left |= static_cast<unsigned long long>(bits) << k0;
+        k0 += kIn;
+    });
+    unsigned short* list = reinterpret_cast<unsigned short*>(dyn + kListOff);
+    {
+        const int lane = threadIdx.x & 31, mine = __popcll(left), upto = warp_incl_scan(mine);
+        int pos = 0;
+        if (lane == 31 && upto) pos = atomicAdd(&sm.nopen[0], upto);
+        pos = __shfl_sync(0xffffffffu, pos, 31) + upto - mine;
+        for (; left; left &= left - 1ull, ++pos)
+            if (pos < kOpenA) list[pos] = static_cast<unsigned short>(t0 + (__ffsll(static_cast<long long>(left)) - 1) * T);
+    }
+    __syncthreads();
+    int c = sm.nopen[0];
+    if (c > kOpenA) return kManyOpen;
+#pragma unroll 1
+    for (int round = 1; c > kMaxOpen; ++round) {  // once more among themselves, with another hash
+        unsigned short* const next = reinterpret_cast<unsigned short*>(dyn + kListOff) + ((round & 1) ? kOpenA : 0);
+        const int room = (round & 1) ? kSelMax - kOpenA : kOpenA;
+        mult = mult * 0x85EBCA77u + 0xC2B2AE3Eu;  // (odd again)
+        if (threadIdx.x == 0) sm.nopen[round & 1] = 0;
+#pragma unroll 1
+        for (int k = threadIdx.x; k < c; k += kST) {
+            const unsigned i = list[k];
+            word[__umulhi(area[i] * mult, nslots)] = static_cast<unsigned short>(i);
         }
         __syncthreads();
-        const int c = sm.nopen[round & 1];
-        if (threadIdx.x == 0) sm.nopen[(round + 1) & 1] = 0;
+#pragma unroll 1
+        for (int k = threadIdx.x; k < c; k += kST) {
+            const unsigned i = list[k], mine = area[i], w = word[__umulhi(mine * mult, nslots)];
+            if (w == i) {
+                ++won;
+            } else if (area[w] != mine) {
+                const int pos = atomicAdd(&sm.nopen[round & 1], 1);
+                if (pos < room) next[pos] = static_cast<unsigned short>(i);
+            }
+        }
+        __syncthreads();
+        list = next;
+        c = sm.nopen[round & 1];
+        if (c > room) return kManyOpen;
+    }
+    // a few are settled by a warp: the first of every cell counts
+    if (threadIdx.x < 32) {
+        const unsigned lane = threadIdx.x, mine = static_cast<int>(lane) < c ? area[list[lane]] : kNoCell;
+        const unsigned same = __match_any_sync(0xffffffffu, mine);
+        won += (static_cast<int>(lane) < c && __ffs(same) - 1 == static_cast<int>(lane)) ? 1u : 0u;
+    }
+    return won;
+}
+
+// kHash where many cells share slots: rounds with other hashes until few points
+// are undecided (every round decides a cell at least).
+template <bool SM, int T>
+__device__ __noinline__ unsigned count_open(int n, const PassGrid* pg, int t0) {
+    uint32_t* const area = pass_area<SM>();
+    unsigned short* const word = reinterpret_cast<unsigned short*>(area + n);
+    unsigned short* const list = reinterpret_cast<unsigned short*>(dyn + kListOff);
+    SmallSmem& sm = smem();
+    const unsigned nslots = pg->nslots;
+    unsigned mult = 0x27D4EB2Fu, won = 0;
+    unsigned long long open = ~0ull;  // bit k: point t0 + k T is undecided
+#pragma unroll 1
+    for (int round = 0; round < n; ++round) {
+        __syncthreads();
+        if (threadIdx.x == 0) sm.nopen[0] = 0;
+#pragma unroll 1
+        for (int k = 0, i = t0; i < n; ++k, i += T)
+            if (((open >> k) & 1ull) && area[i] != kNoCell)
+                word[__umulhi(area[i] * mult, nslots)] = static_cast<unsigned short>(i);
+        __syncthreads();
+        unsigned long long left = 0;
+#pragma unroll 1
+        for (int k = 0, i = t0; i < n; ++k, i += T)
+            if (((open >> k) & 1ull) && area[i] != kNoCell) {
+                const unsigned w = word[__umulhi(area[i] * mult, nslots)];
+                if (w == static_cast<unsigned>(i)) ++won;
+                else if (area[w] != area[i]) left |= 1ull << k;
+            }
+        open = left;
+        for (; left; left &= left - 1ull) {
+            const int pos = atomicAdd(&sm.nopen[0], 1);
+            if (pos < kMaxOpen) list[pos] = static_cast<unsigned short>(t0 + (__ffsll(static_cast<long long>(left)) - 1) * T);
+        }
+        __syncthreads();
+        const int c = sm.nopen[0];
         if (c <= kMaxOpen) {
             if (static_cast<int>(threadIdx.x) < c) {
-                const unsigned mine = area[open_list[threadIdx.x]];
+                const unsigned mine = area[list[threadIdx.x]];
                 bool seen = false;
-                for (int k = 0; k < static_cast<int>(threadIdx.x) && !seen; ++k) seen = area[open_list[k]] == mine;
+                for (int k = 0; k < static_cast<int>(threadIdx.x) && !seen; ++k) seen = area[list[k]] == mine;
                 won += seen ? 0u : 1u;
             }
             break;
         }
-        __syncthreads();
-        open = left;
         mult = mult * 0x85EBCA77u + 0xC2B2AE3Eu;  // (odd again)
-        for (; left; left &= left - 1ull) {
-            const int i = t0 + (__ffsll(static_cast<long long>(left)) - 1) * T;
-            word[__umulhi(area[i] * mult, nslots)] = static_cast<unsigned short>(i);
-        }
-        __syncthreads();
     }
     return won;
 }
 
 // kIndex: the number of points whose voxel was new; nslots words, more than points.
-template <bool SM>
-__device__ __noinline__ unsigned count_index(const float4* src, int n, const PassGrid* pg, int t0, int T) {
+template <bool SM, int T>
+__device__ __noinline__ unsigned count_index(const float4* src, int n, const PassGrid* pg, int t0) {
     uint32_t* const area = pass_area<SM>();
     const Grid& G = pg->bg.g;
     const unsigned nslots = pg->nslots;
@@ -436,10 +518,14 @@ __device__ __noinline__ unsigned count_index(const float4* src, int n, const Pas
     return fresh;
 }
 
-template <bool SM>
-__device__ __forceinline__ unsigned count_pass(const float4* stg, int n, const PassGrid* pg, int t0, int T) {
-    if (pg->mode == kDirect || pg->mode == kHash) return count_cells<SM>(stg, n, pg, t0, T);
-    if (pg->mode == kIndex) return count_index<SM>(stg, n, pg, t0, T);
+// The voxels of a size that this thread's points (t0, t0 + T, ...) count.
+template <bool SM, int T>
+__device__ __forceinline__ unsigned count_pass(const float4* stg, int n, const PassGrid* pg, int t0) {
+    if (pg->mode == kDirect || pg->mode == kHash) {
+        const unsigned won = count_cells<SM, T>(stg, n, pg, t0);
+        return (won != kManyOpen) ? won : count_open<SM, T>(n, pg, t0);
+    }
+    if (pg->mode == kIndex) return count_index<SM, T>(stg, n, pg, t0);
     return 0u;
 }
 
@@ -801,7 +887,7 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                                           lane < 3 ? next_size(sv, hi, up, 0.0f) : next_size(lo, sv, false, 0.0f),
                                           P.aspect, n, area_words);
                             if (!pg.bg.ok) sm.acc_err = 1u;
-                            const unsigned won = __reduce_add_sync(0xffffffffu, count_pass<true>(pts, n, &pg, t0, T));
+                            const unsigned won = __reduce_add_sync(0xffffffffu, count_pass<true, T>(pts, n, &pg, t0));
                             if (lane == 0) sm.wcnt[par][wid] = won;
                             __syncthreads();
                             const int K = static_cast<int>(
@@ -937,8 +1023,8 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                         }
                         __syncthreads();
                         if (!sm.go) break;
-                        unsigned won = in_smem ? count_pass<true>(pts, n, sm.pg, tid, kST)
-                                               : count_pass<false>(stg, n, sm.pg, tid, kST);
+                        unsigned won = in_smem ? count_pass<true, kST>(pts, n, sm.pg, tid)
+                                               : count_pass<false, kST>(stg, n, sm.pg, tid);
                         won = __reduce_add_sync(0xffffffffu, won);
                         if (lane == 0) sm.wcnt[0][wid] = won;
                         __syncthreads();

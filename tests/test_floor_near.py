@@ -16,10 +16,10 @@ def fma(a, b, c):
 
 def fast_floor(x, v, amb):
     r = F(1) / v
-    s = x * r + MAGIC
+    s = fma(x, r, np.full_like(x, MAGIC))
     k = s - MAGIC
     rem = fma(-k, v, x)
-    away = np.abs(rem) > (np.abs(k) + F(2.0**-70)) * amb
+    away = np.abs(rem) > fma(np.abs(k), amb, amb * F(2.0**-70))
     t = s.view(np.int32) + (rem.view(np.int32) >> 31) - 0x4B400000
     kb = k.view(np.int32)
     p = (np.where(k > 0, kb - 1, kb) & 0x7F800000).astype(np.int32).view(F)

@@ -111,3 +111,10 @@ def test_large_forms_and_batches(hv, ctx):
     check(hv, ctx, [lattice(30000, 0.5, 9)], [[5000, 64]])
     clouds = [scenes.uniform_box(k, 10 + k) for k in (1, 40, 700, 2500, 4096)] + [lattice(1500, 0.125, 3)]
     check(hv, ctx, clouds, [[max(1, len(c) // 4), max(1, len(c) // 16)] for c in clouds])
+
+
+# most points in a voxel of their own, with few and with many cells per slot of a pass
+@pytest.mark.parametrize("n,m", [(4096, 4000), (9000, 8900), (20000, 19500), (32768, 31000), (32768, 32700)])
+def test_crowded_passes(hv, ctx, n, m):
+    check(hv, ctx, [scenes.uniform_box(n, n)], [[m]], layers=1)
+    check(hv, ctx, [scattered(n, 2000.0, m)], [[m]], layers=1)
