@@ -61,10 +61,15 @@ constexpr size_t kPassSmem = 4 * static_cast<size_t>(kTilePts) + 2 * static_cast
 constexpr int kSelSlots = 8192;    // block-local argmin table of the selection (128 KB + 16 KB list)
 constexpr size_t kSelSmem = static_cast<size_t>(kSelSlots) * 20;  // + the list of keys that go global
 constexpr size_t kWorkSmem = kPassSmem > kSelSmem ? kPassSmem : kSelSmem;
-// Segments from this size are sorted by Morton cell at level 0: their items then
-// hold most of their voxels whole.  (Measured on GB300, 64 LiDAR clouds of
-// 20,000-200,000 points: 4.42 ms sorted from 2^17, 4.19 from 2^16, 4.06 from
-// 2^14 points; smaller segments run on the small-level kernels by default.)
+// Segments from kBucketMin points are sorted by Morton cell at level 0 where the
+// level has kBucketAll points, else from kBucketAlone: their items then hold most
+// of their voxels whole, which pays for the sort (11 us) only where an item has
+// thousands of points.  (Measured on GB300, 64 LiDAR clouds of 20,000-200,000
+// points: 4.42 ms sorted from 2^17, 4.19 from 2^16, 4.06 from 2^14 points; one
+// LiDAR cloud of 60,000 / 100,000 points: 156 / 193 us sorted, 142 / 175 not.
+// Smaller segments run on the small-level kernels by default.)
+constexpr int kBucketAlone = 1 << 17;
+constexpr int kBucketAll = 1 << 19;
 constexpr int kBucketMin = 1 << 14;
 // Loads and probes in flight per thread (the kernel's template arguments,
 // one instantiation per pass shape): with 64 registers a thread (one
@@ -762,16 +767,21 @@ __device__ __noinline__ long long insert_key(unsigned long long* T, int cap_log2
 // the 1M-point room (17 us, 21.5 us before), 2.6 us are the points, 2.2 the
 // list, 1.6 the ownership, 2.5 the global tables, 4 the barrier with the wait
 // for the slowest block, the rest short sections between block barriers.
-// Measured on GB300, whole calls: room of 1M points, four levels 836 -> 770 us,
-// room of 300,007 points, guided 479 -> 422 us, 64 LiDAR clouds, two levels
-// 4.36 -> 3.55 ms, ten served scenes 1.03 -> 0.87 ms.
+// The rest is instruction fetches: a pass goes through its code once per item,
+// and more code costs more than it hides (a second copy of the point loop
+// without range checks, or the first atomics of several units in flight in (c),
+// made whole calls 2 to 4 % slower).
+// Measured on GB300, whole calls: room of 1M points, four levels 836 -> 715 us,
+// room of 300,007 points, guided 479 -> 407 us, 64 LiDAR clouds, two levels
+// 4.36 -> 3.45 ms, ten served scenes 1.03 -> 0.83 ms, one LiDAR cloud of
+// 200,000 / 100,000 / 60,000 points 207 -> 198 / 185 -> 170 / 142 -> 137 us.
 template <int kProbes, bool kOne>
 __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, unsigned long long* tk, uint32_t* dirty,
                                         int X, long long dstride, LayerState* ls, int cslot, SegHdr* sh, GlobalHdr* gh,
                                         bool prepared, float r0, float r1, float r2) {
-    constexpr int kIn = 4;
+    constexpr int kIn = 3;  // units of a step (4: 1 to 3 % slower where an item has 1,300 to 7,000 points, 2: 2 % in a batch)
     constexpr int kPer = kTilePts / kThreads;  // units of a tile per thread
-    static_assert(kPer % kIn == 0 && kPer <= 32, "one bit per unit");
+    static_assert(kPer + kIn <= 32, "one bit per unit");
     Smem& st = smem_state();
     uint32_t* const cell = reinterpret_cast<uint32_t*>(dyn);
     unsigned short* const word = reinterpret_cast<unsigned short*>(cell + kTilePts);
@@ -1115,13 +1125,14 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
         const int32_t* orig_in = (j == 0) ? nullptr : d.orig((j - 1) & 1);
         uint32_t* taken = d.taken(j & 1);
         const long long NL = st.n_level;
-        // level 0: every segment of at least kBucketMin points is sorted by
+        // level 0: every segment of at least bucket_min points is sorted by
         // Morton cell (one cloud: the whole level; a batch: each such segment
         // within its own range)
+        const int bucket_min = NL >= kBucketAll ? kBucketMin : kBucketAlone;
         bool bucketing = false;
         if (j == 0)
 #pragma unroll 1
-            for (int s2 = 0; s2 < S; ++s2) bucketing = bucketing || st.n[s2] >= kBucketMin;
+            for (int s2 = 0; s2 < S; ++s2) bucketing = bucketing || st.n[s2] >= bucket_min;
 
         // ------------------------------------------------ bbox, layout, clears
         // (a later level's box, masks and states were prepared by the previous
@@ -1134,7 +1145,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 const int s = item_range(st, S, it, &a, &b);
                 float mnv[3] = {INFINITY, INFINITY, INFINITY}, mxv[3] = {-INFINITY, -INFINITY, -INFINITY};
                 int bad = 0;
-                const bool place = st.n[s] < kBucketMin;  // (a bucketed segment is placed by its scatter)
+                const bool place = st.n[s] < bucket_min;  // (a bucketed segment is placed by its scatter)
                 for_points(P.points, a, b, [&](int i, const float* p) {
                     if (place) {
                         ord[i] = make_float4(p[0], p[1], p[2], __int_as_float(i));
@@ -1365,7 +1376,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             if (!grid_sync(d, nb, st, TAG(10, j, 0, 0))) return;
         } else if (bucketing) {
             // ------------------------------- bucketing (large clouds of a batch)
-            // The same counting sort per segment of at least kBucketMin points,
+            // The same counting sort per segment of at least bucket_min points,
             // within the segment's range: counts [S][4096] and cursors [S][4096]
             // in the workspace.  A block's items may belong to several
             // segments: the counts are gathered per run of items of one
@@ -1381,7 +1392,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             if (blockIdx.x == 0)  // the boxes of the sorted segments, for their later levels
 #pragma unroll 1
                 for (int s2 = tid; s2 < S; s2 += kThreads)
-                    if (st.n[s2] >= kBucketMin) {
+                    if (st.n[s2] >= bucket_min) {
                         for (int a3 = 0; a3 < 3; ++a3) {
                             d.sh()[s2].b0[a3] = st.mn[s2][a3];
                             d.sh()[s2].b0[3 + a3] = st.mx[s2][a3];
@@ -1396,7 +1407,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             for (int it = blockIdx.x; it < st.items_total; it += nb) {  // (block-uniform)
                 int a, b;
                 const int s = item_range(st, S, it, &a, &b);
-                if (st.n[s] < kBucketMin) continue;
+                if (st.n[s] < bucket_min) continue;
                 if (hs >= 0 && hs != s) {
 #pragma unroll 1
                     for (int k = tid; k < 4096; k += kThreads)
@@ -1421,7 +1432,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
             for (int it = blockIdx.x; it < st.items_total; it += nb) {  // (block-uniform)
                 int a, b;
                 const int s = item_range(st, S, it, &a, &b);
-                if (st.n[s] < kBucketMin) continue;
+                if (st.n[s] < bucket_min) continue;
                 const int li = static_cast<int>((it - static_cast<int>(blockIdx.x)) / static_cast<int>(nb));
                 if (bs != s) {
                     // exclusive prefix of the segment's 4096 counts, from its first position

@@ -295,8 +295,8 @@ template <bool SM, int T>
 __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const PassGrid* pg, int t0) {
     // Points of a group: more of them cost padding in the last group and code (16 / 8 /
     // 4 / 2 / 1 on 16 CTAs, LiDAR chain of 20,876 points: 343 / 291 / 275 / 288 / 320 us)
-    constexpr int kIn = (SM && T != kST) ? 2 : 4;
-    static_assert(64 % kIn == 0 && kSmallMax <= 64 * kST, "one bit per point of a thread: n <= 64 T");
+    constexpr int kIn = (SM && T != kST) ? 3 : 4;
+    static_assert(kSmallMax <= 64 * kST, "one bit per point of a thread: n <= 64 T");
     uint32_t* const area = pass_area<SM>();
     unsigned short* const word = reinterpret_cast<unsigned short*>(area + n);
     const bool hash = pg->mode == kHash;

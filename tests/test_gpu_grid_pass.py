@@ -89,3 +89,25 @@ def test_passes(hv, ctx, cloud, shape):
                 for l in range(p.layers):
                     why = G.traces_equal(tr[(j * len(clouds) + s) * p.layers + l], tro[j][l])
                     assert why is None, (s, j, l, why)
+
+
+# a level one point short of the size from which its short segments are sorted, and at it
+@pytest.mark.parametrize("total", [(1 << 19) - 1, 1 << 19])
+def test_sort_line(hv, total):
+    short = [scenes.room_scene(n, seed=n) for n in (16383, 16384, 16385)] + [scenes.uniform_box(5, 1)]
+    clouds = short + [scenes.uniform_box(total - sum(len(c) for c in short), 2)]
+    clouds = [np.ascontiguousarray(c, dtype=np.float32) for c in clouds]
+    levels = [[len(c) // 4] for c in clouds]
+    want = G.oracle_many(clouds, levels)
+    pts, offs = scenes.concat(clouds)
+    c = hv.Context(total, len(clouds))
+    try:
+        c.set_tuning(small_points=0, solo_points=0)
+        m = np.array(levels, dtype=np.int64).T
+        out = hv.hav_sample_batched(c, torch.from_numpy(pts).cuda(), offs, m, hv.params())[0].cpu().numpy()
+        assert hv.hav_status_get(c, len(clouds))[0] == 0
+    finally:
+        c.close()
+    for s, (res, _) in enumerate(want):
+        a = int(m[0, :s].sum())
+        assert np.array_equal(out[a:a + m[0, s]], res[0]), s
