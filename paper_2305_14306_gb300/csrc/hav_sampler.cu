@@ -763,17 +763,19 @@ __device__ __noinline__ long long insert_key(unsigned long long* T, int cap_log2
 // range checks, no division, no probing), the ownership test one table look-up
 // per axis instead of its arithmetic per key, and the global tables one round
 // trip where a bit stands for a cell.  The next pass's grids are ready before a
-// pass starts (item_grids).  A pass is bound by latency: of a level-0 pass of
-// the 1M-point room (17 us, 21.5 us before), 2.6 us are the points, 2.2 the
-// list, 1.6 the ownership, 2.5 the global tables, 4 the barrier with the wait
-// for the slowest block, the rest short sections between block barriers.
-// The rest is instruction fetches: a pass goes through its code once per item,
-// and more code costs more than it hides (a second copy of the point loop
+// pass starts (item_grids).  A level-0 pass of the 1M-point room (16 us, 21.5 us
+// before) is bound by latency: 2.6 us are the points, 2.2 the list, 1.6 the
+// ownership, 2.5 the global tables, 4 the barrier with the wait for the slowest
+// block, the rest short sections between block barriers.  In a batch of 7 M points
+// (50 us a pass) the points take 17 us, the memory's rate for 112 MB, the list 15,
+// the ownership 4, the tables 8.
+// A pass goes through its code once per item, and more code costs more than it
+// hides (a second copy of the point loop
 // without range checks, or the first atomics of several units in flight in (c),
 // made whole calls 2 to 4 % slower).
-// Measured on GB300, whole calls: room of 1M points, four levels 836 -> 715 us,
-// room of 300,007 points, guided 479 -> 407 us, 64 LiDAR clouds, two levels
-// 4.36 -> 3.45 ms, ten served scenes 1.03 -> 0.83 ms, one LiDAR cloud of
+// Measured on GB300, whole calls: room of 1M points, four levels 1,029 -> 854 us,
+// room of 300,007 points, guided 495 -> 417 us, 64 LiDAR clouds, two levels
+// 4.27 -> 3.33 ms, ten served scenes 1.03 -> 0.81 ms, one LiDAR cloud of
 // 200,000 / 100,000 / 60,000 points 207 -> 198 / 185 -> 170 / 142 -> 137 us.
 template <int kProbes, bool kOne>
 __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, unsigned long long* tk, uint32_t* dirty,
@@ -854,6 +856,13 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
             }
             // (a) cells and indices
             unsigned mult = 0x9E3779B1u;
+            // (one candidate's, in registers: the stores to the words could change ig)
+            const bool hash0 = ig[0].mode == kCountHash;
+            const unsigned nslots0 = ig[0].nslots;
+            auto word_of = [&](unsigned cn, int c) {
+                const bool h = kOne ? hash0 : ig[c].mode == kCountHash;
+                return c * words + (h ? __umulhi(cn * mult, kOne ? nslots0 : ig[c].nslots) : cn);
+            };
             {
                 CellMap map(ig[0].bg);
                 int c1 = 0;
@@ -885,13 +894,10 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
 #pragma unroll
                     for (int k = 0; k < kIn; ++k) {
                         const int w = w0 + k * kThreads;
-                        const ItemGrid& g = ig[cc[k]];
-                        if (__float_as_int(q[k].w) < 0 || (!kOne && g.mode == kCountNone)) cn[k] = kNoCell;  // taken
+                        if (__float_as_int(q[k].w) < 0 || (!kOne && ig[cc[k]].mode == kCountNone)) cn[k] = kNoCell;  // taken
                         if (w < units) {
                             cell[w] = cn[k];
-                            if (cn[k] != kNoCell)
-                                word[cc[k] * words + (g.mode == kCountHash ? __umulhi(cn[k] * mult, g.nslots) : cn[k])] =
-                                    static_cast<unsigned short>(w);
+                            if (cn[k] != kNoCell) word[word_of(cn[k], cc[k])] = static_cast<unsigned short>(w);
                         }
                     }
                 }
@@ -914,11 +920,7 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
 #pragma unroll
                     for (int k = 0; k < kIn; ++k) {
                         x[k] = -1;
-                        if (cn[k] != kNoCell) {
-                            const int c = kOne ? 0 : (w0 + k * kThreads) / L;
-                            x[k] = word[c * words +
-                                        (ig[c].mode == kCountHash ? __umulhi(cn[k] * mult, ig[c].nslots) : cn[k])];
-                        }
+                        if (cn[k] != kNoCell) x[k] = word[word_of(cn[k], kOne ? 0 : (w0 + k * kThreads) / L)];
                     }
                     int sum = 0;
 #pragma unroll
