@@ -229,8 +229,8 @@ typedef struct {
                                 allocate a larger one (it first waits for the
                                 device); no sampling call allocates */
     int32_t pass_shape;      /* the grid-wide kernel's instantiation: points each
-                                thread loads ahead in a pass and global probes it
-                                keeps in flight, 0: (2, 1) (default), 1: (1, 1),
+                                thread loads ahead in the selection and global
+                                probes it keeps in flight in a pass and there, 0: (2, 1) (default), 1: (1, 1),
                                 2: (2, 2), 3: (4, 1) */
 } hav_tuning;
 

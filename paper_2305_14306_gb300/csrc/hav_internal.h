@@ -46,8 +46,8 @@ constexpr int kChunkMin = 64;              // default smallest work item (points
 constexpr int kSmallMax = 32768;           // largest level the cluster kernel takes (points)
 constexpr int kLocalItems = 8;             // work items one block can own in a level
 // Pass shapes of the grid kernel (template instantiations): points each thread
-// loads ahead in a bisection or selection pass, and first probes of the
-// global flush it keeps in flight.  Shape 0 is the default.
+// loads ahead in the selection, and probes of the global tables it keeps in
+// flight in a bisection pass and there.  Shape 0 is the default.
 constexpr int kPassShapes = 4;
 
 constexpr unsigned long long kEmptyKey = ~0ull;  // valid keys use 63 bits

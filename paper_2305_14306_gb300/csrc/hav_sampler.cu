@@ -71,11 +71,10 @@ constexpr size_t kWorkSmem = kPassSmem > kSelSmem ? kPassSmem : kSelSmem;
 constexpr int kBucketAlone = 1 << 17;
 constexpr int kBucketAll = 1 << 19;
 constexpr int kBucketMin = 1 << 14;
-// Loads and probes in flight per thread (the kernel's template arguments,
-// one instantiation per pass shape): with 64 registers a thread (one
-// 1024-thread block per SM), deeper batches spill more than they hide
-// (measured on GB300: 4 and 2 made the 1M-point chain 5 % slower than the
-// default 2 and 1).
+// Loads (of the selection) and probes in flight per thread (the kernel's
+// template arguments, one instantiation per pass shape).  More of them is more
+// code than it hides latency: with twice the probes whole calls were 2 to 5 %
+// slower on GB300, four loads were within 0.3 % of the default two.
 template <int IF, int PR>
 struct PassShape {
     static constexpr int kInFlight = IF;  // points loaded ahead per thread
@@ -770,9 +769,8 @@ __device__ __noinline__ long long insert_key(unsigned long long* T, int cap_log2
 // (50 us a pass) the points take 17 us, the memory's rate for 112 MB, the list 15,
 // the ownership 4, the tables 8.
 // A pass goes through its code once per item, and more code costs more than it
-// hides (a second copy of the point loop
-// without range checks, or the first atomics of several units in flight in (c),
-// made whole calls 2 to 4 % slower).
+// hides (a second copy of the point loop without range checks, or the first
+// atomics of several units in flight in (c), made whole calls 2 to 4 % slower).
 // Measured on GB300, whole calls: room of 1M points, four levels 1,029 -> 854 us,
 // room of 300,007 points, guided 495 -> 417 us, 64 LiDAR clouds, two levels
 // 4.27 -> 3.33 ms, ten served scenes 1.03 -> 0.81 ms, one LiDAR cloud of
@@ -2083,18 +2081,23 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 if (tid < S) st.cprefix[tid] = cpre;
                 if (tid == 0) st.cprefix[S] = ctot;
                 __syncthreads();
+                // a warp per candidate, the segment's candidates split over its lanes
+                // (one thread each took 27 us for the 836 of 856,000 voxels, half of
+                // the phase's time in a usual layer)
 #pragma unroll 1
-                for (long long w = gtid; w < ctot; w += gstride) {
+                for (int w = (tid >> 5) * static_cast<int>(nb) + static_cast<int>(blockIdx.x); w < ctot;
+                     w += (kThreads / 32) * static_cast<int>(nb)) {
                     const int s = find_seg(st.cprefix, S, w);
-                    const int jdx = static_cast<int>(w) - st.cprefix[s];
+                    const int jdx = w - st.cprefix[s];
                     const int cs = st.cprefix[s + 1] - st.cprefix[s];
                     const Cand* base = d.cand() + st.cand_off[s];
                     const unsigned long long hj = base[jdx].h;
                     int rank = 0;
-#pragma unroll 1
-                    for (int k = 0; k < cs; ++k) rank += (base[k].h < hj) ? 1 : 0;
+#pragma unroll 4
+                    for (int k = tid & 31; k < cs; k += 32) rank += (base[k].h < hj) ? 1 : 0;
+                    rank = __reduce_add_sync(0xffffffffu, rank);
                     const int r = st.ml[s] - static_cast<int>(ls[s].below);
-                    if (rank < r) mark_taken(taken, ord, d.posof(), static_cast<int>(base[jdx].g));
+                    if ((tid & 31) == 0 && rank < r) mark_taken(taken, ord, d.posof(), static_cast<int>(base[jdx].g));
                 }
                 int sf = 0;
                 if (tid < S && (st.flags[tid] & F_ACTIVE) && st.kstar[tid] < st.ml[tid]) sf = 1;

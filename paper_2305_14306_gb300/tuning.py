@@ -10,9 +10,9 @@ A context's knobs (``hav_tuning`` in include/hav.h) that the tuner searches:
 * ``table_log2`` -- the hash-table load factor: a segment's voxel table has
   nextpow2(2^f n) slots for n points (f = 1, 2, 3: at most 1/2, 1/4, 1/8 full;
   a flush waits for its longest probe chain, so emptier tables can pay);
-* ``pass_shape`` -- points each thread loads ahead and global probes it keeps
-  in flight in a pass, one instantiation of the grid kernel each (the block
-  shape itself is fixed: one 1024-thread block per SM);
+* ``pass_shape`` -- points each thread loads ahead (selection) and global probes it keeps
+  in flight, one instantiation of the grid kernel each (the block
+  shape itself is fixed: one 512-thread block per SM);
 * ``small_points`` -- the level size up to which levels run on thread-block
   clusters (0: never).
 
