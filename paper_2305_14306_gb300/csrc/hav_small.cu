@@ -60,7 +60,7 @@ constexpr int kSelMax = 8192;    // slots of a CTA's part of the selection table
 constexpr int kMaxQ = 16;        // largest cluster
 constexpr int kCutBits = 6;      // cut-off histogram over the top priority bits
 constexpr int kCutBins = 1 << kCutBits;
-constexpr int kOpenA = kSelMax / 4 * 3;  // undecided points of a pass that are listed (in later rounds, alternately the rest)
+constexpr int kOpenA = kSelMax / 8 * 7;  // undecided points of a pass that are listed (in later rounds, alternately the rest)
 constexpr unsigned kManyOpen = 0xffffffffu;
 constexpr int kMaxOpen = 32;     // undecided points of a pass that a warp compares with one another
 constexpr int kCandAll = 1024;   // boundary-bin candidates of the cluster that every CTA receives
@@ -289,6 +289,64 @@ __device__ __forceinline__ uint32_t* pass_area() {
 // The counting functions are not inlined: each gets the whole register budget
 // of a thread (64) instead of what the kernel around it leaves.
 
+// The points t0 + b T of a thread's set bits b to the list, of which the first
+// `room` are kept (whole warps; one atomic a warp).
+__device__ __noinline__ void append_open(unsigned long long bits, int t0, int T, unsigned short* list, int room) {
+    SmallSmem& sm = smem();
+    const int mine = __popcll(bits), upto = warp_incl_scan(mine);
+    int pos = 0;
+    if ((threadIdx.x & 31) == 31 && upto) pos = atomicAdd(&sm.nopen[0], upto);
+    pos = __shfl_sync(0xffffffffu, pos, 31) + upto - mine;
+    for (; bits; bits &= bits - 1ull, ++pos)
+        if (pos < room) list[pos] = static_cast<unsigned short>(t0 + (__ffsll(static_cast<long long>(bits)) - 1) * T);
+}
+
+// The cells of the c points listed in `list` that this thread's count: rounds
+// among themselves with other hashes (what a round leaves goes to `other`, and
+// to and fro), the last few by a warp.  In every thread kManyOpen where a round
+// leaves too many.
+__device__ __noinline__ unsigned settle_open(const uint32_t* area, unsigned short* word, unsigned nslots, int c,
+                                             unsigned short* list, int list_room, unsigned short* other, int other_room) {
+    SmallSmem& sm = smem();
+    unsigned mult = 0xB7A56463u, won = 0;
+#pragma unroll 1
+    for (int round = 1; c > kMaxOpen; ++round) {
+        mult = mult * 0x85EBCA77u + 0xC2B2AE3Eu;  // (odd again)
+        if (threadIdx.x == 0) sm.nopen[round & 1] = 0;
+#pragma unroll 1
+        for (int k = threadIdx.x; k < c; k += kST) {
+            const unsigned i = list[k];
+            word[__umulhi(area[i] * mult, nslots)] = static_cast<unsigned short>(i);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int k = threadIdx.x; k < c; k += kST) {
+            const unsigned i = list[k], mine = area[i], w = word[__umulhi(mine * mult, nslots)];
+            if (w == i) {
+                ++won;
+            } else if (area[w] != mine) {
+                const int pos = atomicAdd(&sm.nopen[round & 1], 1);
+                if (pos < other_room) other[pos] = static_cast<unsigned short>(i);
+            }
+        }
+        __syncthreads();
+        c = sm.nopen[round & 1];
+        if (c > other_room) return kManyOpen;
+        unsigned short* const l = list;
+        list = other;
+        other = l;
+        const int r = list_room;
+        list_room = other_room;
+        other_room = r;
+    }
+    if (threadIdx.x < 32) {  // the first of every cell counts
+        const unsigned lane = threadIdx.x, mine = static_cast<int>(lane) < c ? area[list[lane]] : kNoCell;
+        const unsigned same = __match_any_sync(0xffffffffu, mine);
+        won += (static_cast<int>(lane) < c && __ffs(same) - 1 == static_cast<int>(lane)) ? 1u : 0u;
+    }
+    return won;
+}
+
 // kDirect and kHash: the cells this thread's points (t0, t0 + T, ...) stand for.  The area holds
 // the points' cell numbers and nslots 16-bit words behind them.
 template <bool SM, int T>
@@ -301,7 +359,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
     unsigned short* const word = reinterpret_cast<unsigned short*>(area + n);
     const bool hash = pg->mode == kHash;
     const unsigned nslots = pg->nslots;
-    unsigned mult = 0x9E3779B1u;
+    const unsigned mult = 0x9E3779B1u;
     SmallSmem& sm = smem();
     if (threadIdx.x == 0) sm.nopen[0] = 0;
     // group(i0, all): the points i0, i0 + T, ... of which `all`, or those below n, are there.
@@ -377,52 +435,27 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
         left |= static_cast<unsigned long long>(bits) << k0;
         k0 += kIn;
     });
-    unsigned short* list = reinterpret_cast<unsigned short*>(dyn + kListOff);
-    {
-        const int lane = threadIdx.x & 31, mine = __popcll(left), upto = warp_incl_scan(mine);
-        int pos = 0;
-        if (lane == 31 && upto) pos = atomicAdd(&sm.nopen[0], upto);
-        pos = __shfl_sync(0xffffffffu, pos, 31) + upto - mine;
-        for (; left; left &= left - 1ull, ++pos)
-            if (pos < kOpenA) list[pos] = static_cast<unsigned short>(t0 + (__ffsll(static_cast<long long>(left)) - 1) * T);
-    }
+    unsigned short* const list = reinterpret_cast<unsigned short*>(dyn + kListOff);
+    append_open(left, t0, T, list, kOpenA);
     __syncthreads();
     int c = sm.nopen[0];
-    if (c > kOpenA) return kManyOpen;
-#pragma unroll 1
-    for (int round = 1; c > kMaxOpen; ++round) {  // once more among themselves, with another hash
-        unsigned short* const next = reinterpret_cast<unsigned short*>(dyn + kListOff) + ((round & 1) ? kOpenA : 0);
-        const int room = (round & 1) ? kSelMax - kOpenA : kOpenA;
-        mult = mult * 0x85EBCA77u + 0xC2B2AE3Eu;  // (odd again)
-        if (threadIdx.x == 0) sm.nopen[round & 1] = 0;
-#pragma unroll 1
-        for (int k = threadIdx.x; k < c; k += kST) {
-            const unsigned i = list[k];
-            word[__umulhi(area[i] * mult, nslots)] = static_cast<unsigned short>(i);
-        }
+    unsigned more;
+    if (c <= kOpenA) {
+        more = settle_open(area, word, nslots, c, list, kOpenA, list + kOpenA, kSelMax - kOpenA);
+    } else {
+        // too many for the list (levels near 32,768 points in about as many cells):
+        // half of the words, which are done with, take it
+        const int half = static_cast<int>(nslots / 2);
         __syncthreads();
-#pragma unroll 1
-        for (int k = threadIdx.x; k < c; k += kST) {
-            const unsigned i = list[k], mine = area[i], w = word[__umulhi(mine * mult, nslots)];
-            if (w == i) {
-                ++won;
-            } else if (area[w] != mine) {
-                const int pos = atomicAdd(&sm.nopen[round & 1], 1);
-                if (pos < room) next[pos] = static_cast<unsigned short>(i);
-            }
-        }
+        if (threadIdx.x == 0) sm.nopen[0] = 0;
         __syncthreads();
-        list = next;
-        c = sm.nopen[round & 1];
-        if (c > room) return kManyOpen;
+        append_open(left, t0, T, word + half, half);
+        __syncthreads();
+        c = sm.nopen[0];
+        if (c > half) return kManyOpen;
+        more = settle_open(area, word, half, c, word + half, half, list, kSelMax);
     }
-    // a few are settled by a warp: the first of every cell counts
-    if (threadIdx.x < 32) {
-        const unsigned lane = threadIdx.x, mine = static_cast<int>(lane) < c ? area[list[lane]] : kNoCell;
-        const unsigned same = __match_any_sync(0xffffffffu, mine);
-        won += (static_cast<int>(lane) < c && __ffs(same) - 1 == static_cast<int>(lane)) ? 1u : 0u;
-    }
-    return won;
+    return (more != kManyOpen) ? won + more : kManyOpen;
 }
 
 // kHash where many cells share slots: rounds with other hashes until few points
