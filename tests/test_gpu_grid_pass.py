@@ -111,3 +111,22 @@ def test_sort_line(hv, total):
     for s, (res, _) in enumerate(want):
         a = int(m[0, :s].sum())
         assert np.array_equal(out[a:a + m[0, s]], res[0]), s
+
+
+# candidates of the bin that the cut-off falls in: none, one, up to a warp's lanes and many more, in several segments
+@pytest.mark.parametrize("sizes", [[900], [40_000], [150_000], [70_000, 300, 33_000]])
+@pytest.mark.parametrize("part", [1, 2, 5, 97])
+def test_cut_off(hv, ctx, sizes, part):
+    clouds = [np.ascontiguousarray(scenes.uniform_box(n, seed=n), dtype=np.float32) for n in sizes]
+    levels = [[max(1, len(c) * 6 // 10 // part)] for c in clouds]
+    kw = dict(layers=1, fixed_s=0.3)  # nearly every point in a voxel of its own
+    want = G.oracle_many(clouds, levels, kw)
+    pts, offs = scenes.concat(clouds)
+    ctx.set_tuning(nblocks=0)
+    ctx.set_tuning(small_points=0, solo_points=0, pass_shape=0)
+    m = np.array(levels, dtype=np.int64).T
+    out = hv.hav_sample_batched(ctx, torch.from_numpy(pts).cuda(), offs, m, hv.params(**kw))[0].cpu().numpy()
+    assert hv.hav_status_get(ctx, len(clouds))[0] == 0
+    for s, (res, _) in enumerate(want):
+        a = int(m[0, :s].sum())
+        assert np.array_equal(out[a:a + m[0, s]], res[0]), s
