@@ -137,8 +137,16 @@ __device__ __forceinline__ bool make_grid_axis(float s, float r, float mn, Grid*
     return floor_div(mn, v, &g->fmin[a]);
 }
 
+// Up to this many cells from the origin the loops below find a cell without a
+// division: r = __fdividef(1, v) is within 2 units of its last place of 1 / v, a
+// relative 2^-22, so that x * r, rounded to an integer, is within 0.82 of x / v
+// (0.5 for the integer, 0.25 for r, 0.07 where the product is rounded first).
+// From 2^21 on it is not within 1, and from 2^22 on kMagic below rounds to even
+// integers.
+constexpr float kFarCells = 1048576.0f;  // 2^20
+
 // floor(RN(x / v)) without a division.  k is an integer within 1 of x / v (the
-// nearest to x * r for any r close to 1 / v), |k| < 2^22; rem = x - k v is then
+// nearest to x * r for any r close to 1 / v), |k| < kFarCells; rem = x - k v is then
 // exact: a multiple of ulp(v) / 2 (or x itself, k = 0) of size below 2 v, and
 // fma rounds once.  Away from the integer, |x / v - k| > |k| 2^-23, RN(x / v)
 // lies on the side of k that rem's sign tells.  Near it, RN(x / v) >= k exactly
@@ -146,7 +154,7 @@ __device__ __forceinline__ bool make_grid_axis(float s, float r, float mn, Grid*
 // (a tie goes to k, whose last bit is 0), k - 2^(e - 24) with e the exponent of
 // that number (k > 0) or of k (k < 0).  Range of v: floor_cells' caller.
 __device__ __forceinline__ float floor_near(float x, float v, float k, float rem) {
-    if (!(fabsf(k) < 4194304.0f) || (k == 0.0f && fabsf(x) <= __fmul_rn(v, 1e-30f) && x != 0.0f))
+    if (!(fabsf(k) < kFarCells) || (k == 0.0f && fabsf(x) <= __fmul_rn(v, 1e-30f) && x != 0.0f))
         return floorf(__fdiv_rn(x, v));  // (out of range, or a quotient that may underflow)
     const int kb = __float_as_int(k);
     const float p = __int_as_float((k > 0.0f ? kb - 1 : kb) & 0x7f800000);  // 2^e (0 for k = 0)
@@ -163,8 +171,9 @@ __device__ __forceinline__ float floor_near(float x, float v, float k, float rem
 struct BoxGrid {
     Grid g;                    // (r = 0: cell_key divides)
     float ra[3];               // 1 / v, approximately
-    int ci[3];                 // -(kMagicBits + floor(mn / v)) per axis (floor_bits)
+    int ci[3];                 // -(kMagicBits + floor(mn / v)) per axis (floor_bits; of no use in a far box)
     float amb;                 // 2^-22 times the largest v: |rem| up to |k| amb (+ amb 2^-70) is near an integer
+                               // (infinite where the box leaves kFarCells: every point is near)
     unsigned nx, nxy;          // cells along x, and in an x-y layer (where `cells` is below 2^32)
     unsigned c0;               // ci[0] + nx ci[1] + nxy ci[2] mod 2^32 (cell_number)
     int ok, fast;              // the grid is representable; every cell index is in range
@@ -175,10 +184,11 @@ constexpr int kMagicBits = 0x4B400000;
 
 // The bits of kMagic + floor(RN(p / v)) per axis for a point of the box of a
 // fast grid; false where an axis is near an integer (one point in 10^4 to 10^5
-// of a scene).  Without conversion or rounding instructions, which run at a
-// fraction of the rate of additions: k = (q + kMagic) - kMagic, and the bits of
-// q + kMagic are kMagicBits + k; six instructions an axis.  (|q| >= 2^22: |k| amb exceeds v / 2, so the
-// near case takes it.)
+// of a scene) or the box is far from the origin (near_width: the division then
+// decides; 2^22 cells away and more, k would be off by more than |k| amb tells).
+// Without conversion or rounding instructions, which run at a fraction of the
+// rate of additions: k = (q + kMagic) - kMagic, and the bits of q + kMagic are
+// kMagicBits + k; six instructions an axis.
 __device__ __forceinline__ bool floor_bits(const float p[3], const float r[3], const float v[3], float amb, int t[3]) {
     const float amb0 = __fmul_rn(amb, 8.4703294725430034e-22f);  // 2^-70 amb
     bool ok = true;
@@ -257,7 +267,7 @@ static __device__ __noinline__ bool box_axis(float s, float r, float mn, float m
     for (int e = 0; e < 2; ++e) {
         const float x = e ? mx : mn;
         const float k = __fsub_rn(__fadd_rn(__fmul_rn(x, rv), kMagic), kMagic);
-        if (normal && fabsf(k) < 2097152.0f) {
+        if (normal && fabsf(k) < kFarCells) {
             f[e] = floor_near(x, v, k, __fmaf_rn(-k, v, x));
         } else if (!floor_div(x, v, &f[e])) {
             return e == 1;  // (mx alone: the grid stands, without a span)
@@ -267,6 +277,12 @@ static __device__ __noinline__ bool box_axis(float s, float r, float mn, float m
     const float u = __fsub_rn(f[1], f[0]);
     if (normal && u >= 0.0f && u < 2097152.0f) *span = static_cast<unsigned>(u) + 1u;
     return true;
+}
+
+// What an axis (box_axis) adds to BoxGrid::amb, the largest of the three times
+// 2^-22: v, or infinity where a cell of the box lies kFarCells from the origin.
+__device__ __forceinline__ float near_width(float v, float f0, unsigned span) {
+    return (fabsf(f0) < kFarCells && fabsf(f0 + static_cast<float>(span)) < kFarCells) ? v : INFINITY;
 }
 
 // key = u_x | u_y << 21 | u_z << 42 with u = floor(x / v) - floor(min / v).

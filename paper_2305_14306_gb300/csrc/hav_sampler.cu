@@ -633,7 +633,8 @@ __device__ __noinline__ void item_grids(int S, unsigned nb, int w0, int li0, int
     const int ci = (fabsf(f0) < 4194304.0f) ? -(kMagicBits + static_cast<int>(f0)) : 0;
     const unsigned part = static_cast<unsigned>(ci) * (ax == 0 ? 1u : (ax == 1 ? nx : nx * ny));
     const unsigned c0 = part + __shfl_sync(0xffffffffu, part, lead + 1) + __shfl_sync(0xffffffffu, part, lead + 2);
-    const float vmax = fmaxf(v, fmaxf(__shfl_sync(0xffffffffu, v, lead + 1), __shfl_sync(0xffffffffu, v, lead + 2)));
+    const float vn = near_width(v, f0, span);
+    const float vmax = fmaxf(vn, fmaxf(__shfl_sync(0xffffffffu, vn, lead + 1), __shfl_sync(0xffffffffu, vn, lead + 2)));
     if (e >= count || lane >= 30) return;
     ItemGrid& g = st.ig[e];
     g.bg.g.v[ax] = v;

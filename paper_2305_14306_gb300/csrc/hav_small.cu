@@ -578,7 +578,8 @@ __device__ __noinline__ void set_grids(int first, int sizes, float sv, const flo
     const int ci = (fabsf(f0) < 4194304.0f) ? -(kMagicBits + static_cast<int>(f0)) : 0;
     const unsigned part = static_cast<unsigned>(ci) * (ax == 0 ? 1u : (ax == 1 ? nx : nx * ny));
     const unsigned c0 = part + __shfl_sync(0xffffffffu, part, lead + 1) + __shfl_sync(0xffffffffu, part, lead + 2);
-    const float vmax = fmaxf(v, fmaxf(__shfl_sync(0xffffffffu, v, lead + 1), __shfl_sync(0xffffffffu, v, lead + 2)));
+    const float vn = near_width(v, f0, span);
+    const float vmax = fmaxf(vn, fmaxf(__shfl_sync(0xffffffffu, vn, lead + 1), __shfl_sync(0xffffffffu, vn, lead + 2)));
     if (o < sizes && lane < 30) {
         PassGrid& g = sm.pg[first + o];
         g.bg.g.v[ax] = v;
