@@ -916,11 +916,11 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                         for (;;) {
                             const PassGrid& pg = sm.pg[cur];
                             const float sv = pg.sv;
+                            const bool fits = pg.bg.ok != 0;  // (alike in every thread)
                             if (wid == kWarps - 1)  // outcome 0: too many voxels, 1: too few
                                 set_grids(2 * (par ^ 1), 2,
                                           lane < 3 ? next_size(sv, hi, up, 0.0f) : next_size(lo, sv, false, 0.0f),
                                           P.aspect, n, area_words);
-                            if (!pg.bg.ok) sm.acc_err = 1u;
                             const unsigned won = __reduce_add_sync(0xffffffffu, count_pass<true, T>(pts, n, &pg, t0));
                             if (lane == 0) sm.wcnt[par][wid] = won;
                             __syncthreads();
@@ -936,7 +936,9 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                                 if (K >= ml) pre = false;
                             }
                             ++t;
-                            if (sm.acc_err) {
+                            // (a pass sets acc_err behind a barrier of its own (count_index), so
+                            // what a warp reads here is this pass's and not a faster warp's next)
+                            if (!fits || sm.acc_err) {
                                 err = HAV_ERR_RANGE;
                                 break;
                             }
