@@ -154,8 +154,8 @@ struct Smem {
     // a bucketed segment (level 0, and for one cloud the levels that keep its
     // order): per work item of the block, the Morton cells [own_lo, own_hi]
     // of the level-0 bucketing (its box own_mn, own_k[a] = 16 / extent) whose
-    // points all lie in the item (own_on); per pass the keys that go to the
-    // global table (rest_n) and the owned ones counted here.  b0_*: one
+    // points all lie in the item (own_on); per pass the undecided units
+    // (rest_n) and the owned ones counted here.  b0_*: one
     // bucketed cloud's level-0 box, kept for its later levels.
     int own_on[kLocalItems], own_lo[kLocalItems], own_hi[kLocalItems], bucketed;
     float own_k[kLocalItems][3], own_mn[kLocalItems][3];
@@ -163,7 +163,7 @@ struct Smem {
     unsigned rest_n;
     unsigned xcnt[kMaxCand];
     int ocnt[kLocalItems];  // owned voxels the selection listed for the classification, per item
-    unsigned gl_n;          // keys of the selection that go to the global table
+    unsigned gl_n;          // units of a pass, or keys of the selection, that go to the global table
     unsigned bh[kHistBins]; // this block's cut-off histogram of a selection (added to the global one once)
     int ntimes;
     int was_clean;
@@ -846,6 +846,7 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
             if (tid == 0) {
                 st.list_n = 0u;
                 st.rest_n = 0u;
+                st.gl_n = 0u;
             }
             if (keys) {
                 __syncthreads();
@@ -971,6 +972,8 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
             int ng = nl;
             // (b) a voxel whose every point lies in Morton cells this item holds whole
             // is counted here (below 256 listed units the test costs about what it saves)
+            // (behind the open units, under a counter of its own: no barrier lies between
+            // the rounds' last look at rest_n and the first append here)
             if (own && nl >= 256) {
                 unsigned mine = 0;
                 for (int k0 = tid - lane; k0 < nl; k0 += kThreads) {  // warp-uniform
@@ -992,8 +995,8 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
                                    static_cast<int>(m >> 16) > st.own_hi[li];
                         }
                     }
-                    const int pos = warp_append(glob, &st.rest_n);
-                    if (pos >= 0) rest[pos] = static_cast<unsigned short>(w);
+                    const int pos = warp_append(glob, &st.gl_n);
+                    if (pos >= 0) rest[nopen + pos] = static_cast<unsigned short>(w);
                     if (kOne) mine += (k < nl && !glob) ? 1u : 0u;
                     else warp_append_keyed(k < nl && !glob, c, st.xcnt);
                 }
@@ -1003,7 +1006,7 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
                 }
                 __syncthreads();
                 gl = rest;
-                ng = static_cast<int>(st.rest_n);
+                ng = nopen + static_cast<int>(st.gl_n);
             } else if (nopen) {
                 for (int k = tid; k < nopen; k += kThreads) list[nl + k] = rest[k];
                 __syncthreads();
