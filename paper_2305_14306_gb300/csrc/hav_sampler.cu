@@ -691,8 +691,21 @@ __device__ __forceinline__ void cell_axes(unsigned c, const ItemGrid& g, unsigne
     u[1] = div_mod(rest, g.bg.nx, g.mx, &u[0]);
 }
 
-// The units of a tile whose cells or keys leave the ranges of pass_items, key
-// by key into the global tables (a function of its own: seldom used).
+// The bit of cell `cell` of a segment's box (at most 64 cells a slot) in a
+// candidate's table; whether it was not set before, and its slot (neighbouring
+// cells in different ones).
+__device__ __forceinline__ bool set_bit(unsigned long long* T, int cap_log2, unsigned cell, long long* slot) {
+    *slot = cell & ((1u << cap_log2) - 1u);
+    const unsigned bit = static_cast<unsigned>(static_cast<unsigned long long>(cell) >> cap_log2);
+    const unsigned m = 1u << (bit & 31u);
+    unsigned* const wd = reinterpret_cast<unsigned*>(T + *slot) + (bit >> 5);
+    return (atomicAnd(wd, ~m) & m) != 0u;
+}
+
+// The units of a tile whose cells or keys leave the ranges of pass_items, point
+// by point into the global tables (a function of its own: seldom used).  One
+// candidate's cells send all candidates of the item here, so a candidate whose
+// table holds bits (snx: alike in every item of the segment) gets bits here too.
 __device__ __noinline__ int pass_keys(const float4* ord, const ItemGrid* ig, int ncand, int a, int ia, int L, int li,
                                       int s, int X, unsigned long long* tk, uint32_t* dirty, long long dstride) {
     Smem& st = smem_state();
@@ -723,8 +736,15 @@ __device__ __noinline__ int pass_keys(const float4* ord, const ItemGrid* ig, int
         bool fr = false;
         long long slot = -1;
         if (in) {
-            slot = find_or_insert(tk + st.tab_off[s] + c * tstride, st.cap_log2[s], key, &fr);
-            if (slot < 0) bad = HAV_ERR_TABLE_FULL;
+            unsigned long long* const T = tk + st.tab_off[s] + c * tstride;
+            if (ig[c].snx) {
+                const unsigned ux = static_cast<unsigned>(key) & 0x1fffffu, uy = static_cast<unsigned>(key >> 21) & 0x1fffffu,
+                               uz = static_cast<unsigned>(key >> 42);
+                fr = set_bit(T, st.cap_log2[s], ux + ig[c].snx * uy + ig[c].snxy * uz, &slot);
+            } else {
+                slot = find_or_insert(T, st.cap_log2[s], key, &fr);
+                if (slot < 0) bad = HAV_ERR_TABLE_FULL;
+            }
         }
         const bool fresh = in && slot >= 0 && fr;
         const int k = warp_append_keyed(fresh, c, st.dcnt[X][li]);
@@ -1013,8 +1033,7 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
                 ng = nl + nopen;
             }
             // (c) the others into the global tables: a bit per cell of the segment's box
-            // where it fits the table's memory (one round trip, no probing; neighbouring
-            // cells in different slots), else the keys
+            // where it fits the table's memory (one round trip, no probing), else the keys
             for (int k0 = tid - lane; k0 < ng; k0 += kProbes * kThreads) {  // warp-uniform
                 unsigned long long key[kProbes];
                 unsigned long long* Tp[kProbes];
@@ -1039,12 +1058,7 @@ __device__ __noinline__ void pass_items(int S, unsigned nb, const float4* ord, u
                         for (int ax = 0; ax < 3; ++ax) u[ax] += static_cast<unsigned>(g.off[ax]);
                         Tp[k2] = Tb + cc[k2] * tstride;
                         if (g.snx) {
-                            const unsigned cell_s = u[0] + g.snx * u[1] + g.snxy * u[2];
-                            slot[k2] = cell_s & ((1u << cap) - 1u);
-                            const unsigned bit = static_cast<unsigned>(static_cast<unsigned long long>(cell_s) >> cap);
-                            const unsigned m = 1u << (bit & 31u);
-                            unsigned* const wd = reinterpret_cast<unsigned*>(Tp[k2] + slot[k2]) + (bit >> 5);
-                            fr[k2] = (atomicAnd(wd, ~m) & m) != 0u;
+                            fr[k2] = set_bit(Tp[k2], cap, u[0] + g.snx * u[1] + g.snxy * u[2], &slot[k2]);
                         } else {
                             key[k2] = static_cast<unsigned long long>(u[0]) | (static_cast<unsigned long long>(u[1]) << 21) |
                                       (static_cast<unsigned long long>(u[2]) << 42);
