@@ -148,7 +148,8 @@ constexpr float kFarCells = 1048576.0f;  // 2^20
 // floor(RN(x / v)) without a division.  k is an integer within 1 of x / v (the
 // nearest to x * r for any r close to 1 / v), |k| < kFarCells; rem = x - k v is then
 // exact: a multiple of ulp(v) / 2 (or x itself, k = 0) of size below 2 v, and
-// fma rounds once.  Away from the integer, |x / v - k| > |k| 2^-23, RN(x / v)
+// fma rounds once.  Away from the integer, |x / v - k| > |k| 2^-24 (half the
+// spacing of binary32 below k at most), RN(x / v)
 // lies on the side of k that rem's sign tells.  Near it, RN(x / v) >= k exactly
 // when x / v is at least the midpoint of k and the binary32 number below it
 // (a tie goes to k, whose last bit is 0), k - 2^(e - 24) with e the exponent of
@@ -172,7 +173,7 @@ struct BoxGrid {
     Grid g;                    // (r = 0: cell_key divides)
     float ra[3];               // 1 / v, approximately
     int ci[3];                 // -(kMagicBits + floor(mn / v)) per axis (floor_bits; of no use in a far box)
-    float amb;                 // 2^-22 times the largest v: |rem| up to |k| amb (+ amb 2^-70) is near an integer
+    float amb;                 // kNear times the largest v: |rem| up to |k| amb (+ amb 2^-70) is near an integer
                                // (infinite where the box leaves kFarCells: every point is near)
     unsigned nx, nxy;          // cells along x, and in an x-y layer (where `cells` is below 2^32)
     unsigned c0;               // ci[0] + nx ci[1] + nxy ci[2] mod 2^32 (cell_number)
@@ -181,9 +182,10 @@ struct BoxGrid {
 };
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: q + kMagic is kMagic + the integer nearest to q for |q| < 2^22
 constexpr int kMagicBits = 0x4B400000;
+constexpr float kNear = 0x1.01p-24f;  // 2^-24 and what the products of the test may lose
 
 // The bits of kMagic + floor(RN(p / v)) per axis for a point of the box of a
-// fast grid; false where an axis is near an integer (one point in 10^4 to 10^5
+// fast grid; false where an axis is near an integer (one point in 10^5 to 10^6
 // of a scene) or the box is far from the origin (near_width: the division then
 // decides; 2^22 cells away and more, k would be off by more than |k| amb tells).
 // Without conversion or rounding instructions, which run at a fraction of the
@@ -280,9 +282,10 @@ static __device__ __noinline__ bool box_axis(float s, float r, float mn, float m
 }
 
 // What an axis (box_axis) adds to BoxGrid::amb, the largest of the three times
-// 2^-22: v, or infinity where a cell of the box lies kFarCells from the origin.
-__device__ __forceinline__ float near_width(float v, float f0, unsigned span) {
-    return (fabsf(f0) < kFarCells && fabsf(f0 + static_cast<float>(span)) < kFarCells) ? v : INFINITY;
+// kNear: v, or infinity where a cell of the box lies `limit` from the origin
+// (kFarCells at most).
+__device__ __forceinline__ float near_width(float v, float f0, unsigned span, float limit = kFarCells) {
+    return (fabsf(f0) < limit && fabsf(f0 + static_cast<float>(span)) < limit) ? v : INFINITY;
 }
 
 // key = u_x | u_y << 21 | u_z << 42 with u = floor(x / v) - floor(min / v).

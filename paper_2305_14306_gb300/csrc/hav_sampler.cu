@@ -649,7 +649,7 @@ __device__ __noinline__ void item_grids(int S, unsigned nb, int w0, int li0, int
         const unsigned long long cells = static_cast<unsigned long long>(nx) * ny * nz;
         const unsigned long long scells = static_cast<unsigned long long>(sx) * sy * sz;
         const unsigned words = static_cast<unsigned>(kPassWords / ncand);
-        g.bg.amb = __fmul_rn(vmax, 2.384185791015625e-07f);  // 2^-22
+        g.bg.amb = __fmul_rn(vmax, kNear);
         g.bg.nx = nx;
         g.bg.nxy = nx * ny;
         g.bg.c0 = c0;

@@ -102,7 +102,7 @@ struct PassGrid {
     float sv;
     int mode;
     unsigned nslots;  // 16-bit words of kDirect and kHash, 32-bit words of kIndex
-    int pad;
+    int far;          // the box leaves kFarLoop: far_cells
 };
 
 struct SmallSmem {
@@ -347,9 +347,47 @@ __device__ __noinline__ unsigned settle_open(const uint32_t* area, unsigned shor
     return won;
 }
 
-// kDirect and kHash: the cells this thread's points (t0, t0 + T, ...) stand for.  The area holds
-// the points' cell numbers and nslots 16-bit words behind them.
+// The first loop of count_cells over a box far from the origin, where a warp
+// seldom has no point near an integer: the cells are divided for without a first
+// look.  (16 CTAs, 20,000 points, voxels 2^18 / 2^22 cells from the origin: 143 / 126
+// us a call, with the second look at every point 235 / 200, near the origin 94.  The
+// loops cost the same at about 2^16 cells.)
+constexpr float kFarLoop = 65536.0f;  // cells from the origin
 template <bool SM, int T>
+__device__ __noinline__ void far_cells(const float4* stg, int n, const PassGrid* pg, unsigned short* word, unsigned mult,
+                                       int t0) {
+    constexpr int kIn = 2;
+    uint32_t* const area = pass_area<SM>();
+    const bool hash = pg->mode == kHash;
+    const unsigned nslots = pg->nslots, nx = pg->bg.nx, nxy = pg->bg.nxy;
+    const float v[3] = {pg->bg.g.v[0], pg->bg.g.v[1], pg->bg.g.v[2]};
+    const float f0[3] = {pg->bg.g.fmin[0], pg->bg.g.fmin[1], pg->bg.g.fmin[2]};
+#pragma unroll 1
+    for (int i0 = t0; i0 < n; i0 += kIn * T) {
+        float4 q[kIn];
+#pragma unroll
+        for (int k = 0; k < kIn; ++k) q[k] = load_point<SM>(stg, min(i0 + k * T, n - 1));
+#pragma unroll
+        for (int k = 0; k < kIn; ++k) {
+            const int i = i0 + k * T;
+            if (i >= n) break;
+            const float p[3] = {q[k].x, q[k].y, q[k].z};
+            unsigned u[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                u[a] = static_cast<unsigned>(static_cast<int>(__fsub_rn(floorf(__fdiv_rn(p[a], v[a])), f0[a])));
+            const unsigned c = u[0] + nx * u[1] + nxy * u[2];
+            const bool in = __float_as_int(q[k].w) >= 0;
+            area[i] = in ? c : kNoCell;
+            if (in) word[hash ? __umulhi(c * mult, nslots) : c] = static_cast<unsigned short>(i);
+        }
+    }
+}
+
+// kDirect and kHash: the cells this thread's points (t0, t0 + T, ...) stand for.  The area holds
+// the points' cell numbers and nslots 16-bit words behind them.  kRare: of a far box (in a
+// function of its own: code beside the loops below costs every pass).
+template <bool SM, int T, bool kRare>
 __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const PassGrid* pg, int t0) {
     // Points of a group: more of them cost padding in the last group and code (16 / 8 /
     // 4 / 2 / 1 on 16 CTAs, LiDAR chain of 20,876 points: 343 / 291 / 275 / 288 / 320 us)
@@ -373,7 +411,9 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
 #pragma unroll 1
         for (; i0 < n; i0 += kIn * T) group(i0, std::false_type{});
     };
-    {
+    if constexpr (kRare) {
+        far_cells<SM, T>(stg, n, pg, word, mult, t0);
+    } else {
         const CellMap cell(pg->bg);
         each([&](int i0, auto all) {
             float4 q[kIn];
@@ -555,7 +595,8 @@ __device__ __noinline__ unsigned count_index(const float4* src, int n, const Pas
 template <bool SM, int T>
 __device__ __forceinline__ unsigned count_pass(const float4* stg, int n, const PassGrid* pg, int t0) {
     if (pg->mode == kDirect || pg->mode == kHash) {
-        const unsigned won = count_cells<SM, T>(stg, n, pg, t0);
+        const unsigned won = (T == kST && pg->far) ? count_cells<SM, kST, true>(stg, n, pg, t0)
+                                                   : count_cells<SM, T, false>(stg, n, pg, t0);
         return (won != kManyOpen) ? won : count_open<SM, T>(n, pg, t0);
     }
     if (pg->mode == kIndex) return count_index<SM, T>(stg, n, pg, t0);
@@ -578,7 +619,7 @@ __device__ __noinline__ void set_grids(int first, int sizes, float sv, const flo
     const int ci = (fabsf(f0) < 4194304.0f) ? -(kMagicBits + static_cast<int>(f0)) : 0;
     const unsigned part = static_cast<unsigned>(ci) * (ax == 0 ? 1u : (ax == 1 ? nx : nx * ny));
     const unsigned c0 = part + __shfl_sync(0xffffffffu, part, lead + 1) + __shfl_sync(0xffffffffu, part, lead + 2);
-    const float vn = near_width(v, f0, span);
+    const float vn = near_width(v, f0, span, kFarLoop);
     const float vmax = fmaxf(vn, fmaxf(__shfl_sync(0xffffffffu, vn, lead + 1), __shfl_sync(0xffffffffu, vn, lead + 2)));
     if (o < sizes && lane < 30) {
         PassGrid& g = sm.pg[first + o];
@@ -598,7 +639,8 @@ __device__ __noinline__ void set_grids(int first, int sizes, float sv, const flo
             g.nslots = direct ? static_cast<unsigned>(cells)
                               : (hashed ? min(words, 4u * static_cast<unsigned>(n))
                                         : min(static_cast<unsigned>(2 * n + 64), area_words));
-            g.bg.amb = __fmul_rn(vmax, 2.384185791015625e-07f);  // 2^-22
+            g.far = isinf(vmax) ? 1 : 0;
+            g.bg.amb = __fmul_rn(vmax, kNear);
             g.bg.nx = nx;
             g.bg.nxy = nx * ny;
             g.bg.c0 = c0;

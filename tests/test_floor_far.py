@@ -13,9 +13,6 @@ F = np.float32
 
 # A grid over a box as the kernels put it together, an axis at a time, and its points' cells.
 CODE = r"""
-#ifndef NEAR_WIDTH
-static inline float near_width(float v, float, unsigned) { return v; }
-#endif
 // out[0]: cells that are not the floor's, out[1]: out of the box, out[2]: taken without a second look
 extern "C" int cells(const float* pts, int n, float s, const float* aspect, long long* out) {
     float mn[3], mx[3];
@@ -35,7 +32,7 @@ extern "C" int cells(const float* pts, int n, float s, const float* aspect, long
     }
     b.cells = static_cast<unsigned long long>(span[0]) * span[1] * span[2];
     if (b.cells >= kNoCell) return 0;
-    b.amb = __fmul_rn(vmax, 2.384185791015625e-07f);
+    b.amb = __fmul_rn(vmax, kNear);
     b.nx = span[0];
     b.nxy = span[0] * span[1];
     b.c0 = static_cast<unsigned>(b.ci[0]) + b.nx * static_cast<unsigned>(b.ci[1]) + b.nxy * static_cast<unsigned>(b.ci[2]);
@@ -67,8 +64,7 @@ extern "C" int cells(const float* pts, int n, float s, const float* aspect, long
 @pytest.fixture(scope="module", params=[-2, -1, 0, 1, 2], ids=lambda u: f"{u:+d} ulp")
 def cells(request, tmp_path_factory):
     text = H.passage("hav_device.cuh", "struct Grid {", "// At most this many voxels are occupied")
-    flags = [f"-DULPS={request.param}"] + (["-DNEAR_WIDTH"] if "near_width" in text else [])
-    lib = H.compile_host(tmp_path_factory.mktemp("cells"), text + CODE, *flags)
+    lib = H.compile_host(tmp_path_factory.mktemp("cells"), text + CODE, f"-DULPS={request.param}")
 
     def run(pts, s, aspect=(1, 1, 1)):
         pts = np.ascontiguousarray(pts, dtype=F)
