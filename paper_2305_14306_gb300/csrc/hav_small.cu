@@ -91,17 +91,27 @@ __host__ __device__ constexpr int qlog2() {
 //            write.  (A bitmap and a table of cell numbers, one shared-memory
 //            atomic per point, took 1.7 to 2.5 times as long: neighbouring
 //            points' atomics meet in one word.)
-//   kIndex   (2^32 cells and more, or a cell index that may be out of range)
-//            open addressing on (16 key bits, point index) with atomics,
-//            compared through the indexed point's key
-enum : int { kSkip = 0, kDirect = 1, kHash = 2, kIndex = 3 };
+//   kWide    (2^32 cells and more, on a cluster) kHash on the cell numbers modulo
+//            2^32.  A point that reads one of its own number compares the cells
+//            themselves (wide_check), a look at the points that share a voxel.
+//            Where the cells differ, all points of the one that the word does not
+//            stand for do so (equal numbers read the same word): they are
+//            collected with their keys, and their distinct keys added.  In a
+//            scan hardly two cells share a number.  (16 CTAs, a LiDAR scan of
+//            24,000 points to 97 of 100, one layer: 217 us by kIndex, 101 so; a
+//            pass 30 us, 17 to 21 by kHash.)
+//   kIndex   (a cell index that may be out of range, more points with a shared
+//            number than are collected, or 2^32 cells on one CTA) open addressing
+//            on (16 key bits, point index) with atomics, compared through the
+//            indexed point's key
+enum : int { kSkip = 0, kDirect = 1, kHash = 2, kWide = 3, kIndex = 4 };
 
 // A pass's size, its grid over the level's box, and how a pass counts it.
 struct PassGrid {
     BoxGrid bg;
     float sv;
     int mode;
-    unsigned nslots;  // 16-bit words of kDirect and kHash, 32-bit words of kIndex
+    unsigned nslots;  // 16-bit words of kDirect, kHash and kWide
     int far;          // the box leaves kFarLoop: far_cells
 };
 
@@ -137,6 +147,7 @@ struct SmallSmem {
     int bin_cnt[kMaxQ];  // records of this CTA's share by owner: counts, then places
     unsigned nlist;           // slots the selection filled
     int nopen[2];             // undecided points of a kHash round, by its parity
+    int ntwin;                // points of cells that share another's number (kWide)
     unsigned own_cand;        // this CTA's boundary-bin candidates, at the front of the slot list
     int cut_bin, cut_below, kstar;
     unsigned eb;
@@ -301,12 +312,70 @@ __device__ __noinline__ void append_open(unsigned long long bits, int t0, int T,
         if (pos < room) list[pos] = static_cast<unsigned short>(t0 + (__ffsll(static_cast<long long>(bits)) - 1) * T);
 }
 
+// The key of a point's cell (a fast grid).
+__device__ __forceinline__ unsigned long long key_of(const float4& q, const BoxGrid& B) {
+    const float p[3] = {q.x, q.y, q.z};
+    int u[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) u[a] = static_cast<int>(__fsub_rn(floorf(__fdiv_rn(p[a], B.g.v[a])), B.g.fmin[a]));
+    return static_cast<unsigned long long>(u[0]) | (static_cast<unsigned long long>(u[1]) << 21) |
+           (static_cast<unsigned long long>(u[2]) << 42);
+}
+
+// kWide: the keys collected, in the room of the received candidates (which the
+// cut-off fills, cluster barriers later).
+__device__ __forceinline__ unsigned long long* twin_keys() {
+    return reinterpret_cast<unsigned long long*>(dyn + kPtsBytes + kTabBytes);
+}
+__device__ __forceinline__ void add_twin(unsigned long long key) {
+    const int pos = atomicAdd(&smem().ntwin, 1);
+    if (pos < kCandAll) twin_keys()[pos] = key;
+}
+
+// kWide, behind a round's reads: of this thread's points that took another's word
+// for their cell's (set bits: point t0 + b T, or the one listed there), those whose
+// cells differ.
+template <bool SM>
+__device__ __noinline__ void wide_check(const float4* stg, const PassGrid* pg, const unsigned short* word, unsigned nslots,
+                                        unsigned mult, unsigned long long bits, int t0, int T, const unsigned short* list) {
+    const uint32_t* const area = pass_area<SM>();
+#pragma unroll 1
+    for (; bits; bits &= bits - 1ull) {
+        int i = t0 + (__ffsll(static_cast<long long>(bits)) - 1) * T;
+        if (list) i = list[i];
+        const float4 a = load_point<SM>(stg, i), b = load_point<SM>(stg, word[__umulhi(area[i] * mult, nslots)]);
+        const unsigned long long key = key_of(a, pg->bg);
+        if (key != key_of(b, pg->bg)) add_twin(key);
+    }
+}
+
+// The cells that this thread counts of those collected; kManyOpen where they are too many.
+__device__ __noinline__ unsigned count_twins() {
+    __syncthreads();
+    const int twins = smem().ntwin;
+    if (twins > kCandAll) return kManyOpen;
+    const unsigned long long* const key = twin_keys();
+    unsigned won = 0;
+#pragma unroll 1
+    for (int k = threadIdx.x; k < twins; k += kST) {
+        bool seen = false;
+#pragma unroll 1
+        for (int e = 0; e < k && !seen; ++e) seen = key[e] == key[k];
+        won += seen ? 0u : 1u;
+    }
+    return won;
+}
+
 // The cells of the c points listed in `list` that this thread's count: rounds
 // among themselves with other hashes (what a round leaves goes to `other`, and
 // to and fro), the last few by a warp.  In every thread kManyOpen where a round
 // leaves too many.
-__device__ __noinline__ unsigned settle_open(const uint32_t* area, unsigned short* word, unsigned nslots, int c,
-                                             unsigned short* list, int list_room, unsigned short* other, int other_room) {
+template <bool SM, bool kRare>
+__device__ __noinline__ unsigned settle_open(const float4* stg, const PassGrid* pg, unsigned short* word, unsigned nslots,
+                                             int c, unsigned short* list, int list_room, unsigned short* other,
+                                             int other_room) {
+    const uint32_t* const area = pass_area<SM>();
+    const bool wide = kRare && pg->mode == kWide;
     SmallSmem& sm = smem();
     unsigned mult = 0xB7A56463u, won = 0;
 #pragma unroll 1
@@ -319,6 +388,8 @@ __device__ __noinline__ unsigned settle_open(const uint32_t* area, unsigned shor
             word[__umulhi(area[i] * mult, nslots)] = static_cast<unsigned short>(i);
         }
         __syncthreads();
+        unsigned long long same = 0;
+        int b = 0;
 #pragma unroll 1
         for (int k = threadIdx.x; k < c; k += kST) {
             const unsigned i = list[k], mine = area[i], w = word[__umulhi(mine * mult, nslots)];
@@ -327,8 +398,12 @@ __device__ __noinline__ unsigned settle_open(const uint32_t* area, unsigned shor
             } else if (area[w] != mine) {
                 const int pos = atomicAdd(&sm.nopen[round & 1], 1);
                 if (pos < other_room) other[pos] = static_cast<unsigned short>(i);
+            } else if (kRare) {
+                same |= 1ull << b;
             }
+            if (kRare) ++b;
         }
+        if (wide) wide_check<SM>(stg, pg, word, nslots, mult, same, threadIdx.x, kST, list);
         __syncthreads();
         c = sm.nopen[round & 1];
         if (c > other_room) return kManyOpen;
@@ -341,7 +416,10 @@ __device__ __noinline__ unsigned settle_open(const uint32_t* area, unsigned shor
     }
     if (threadIdx.x < 32) {  // the first of every cell counts
         const unsigned lane = threadIdx.x, mine = static_cast<int>(lane) < c ? area[list[lane]] : kNoCell;
-        const unsigned same = __match_any_sync(0xffffffffu, mine);
+        unsigned same = __match_any_sync(0xffffffffu, mine);
+        if (wide)
+            same = __match_any_sync(
+                0xffffffffu, static_cast<int>(lane) < c ? key_of(load_point<SM>(stg, list[lane]), pg->bg) : ~0ull);
         won += (static_cast<int>(lane) < c && __ffs(same) - 1 == static_cast<int>(lane)) ? 1u : 0u;
     }
     return won;
@@ -358,7 +436,7 @@ __device__ __noinline__ void far_cells(const float4* stg, int n, const PassGrid*
                                        int t0) {
     constexpr int kIn = 2;
     uint32_t* const area = pass_area<SM>();
-    const bool hash = pg->mode == kHash;
+    const bool hash = pg->mode != kDirect;
     const unsigned nslots = pg->nslots, nx = pg->bg.nx, nxy = pg->bg.nxy;
     const float v[3] = {pg->bg.g.v[0], pg->bg.g.v[1], pg->bg.g.v[2]};
     const float f0[3] = {pg->bg.g.fmin[0], pg->bg.g.fmin[1], pg->bg.g.fmin[2]};
@@ -376,7 +454,7 @@ __device__ __noinline__ void far_cells(const float4* stg, int n, const PassGrid*
 #pragma unroll
             for (int a = 0; a < 3; ++a)
                 u[a] = static_cast<unsigned>(static_cast<int>(__fsub_rn(floorf(__fdiv_rn(p[a], v[a])), f0[a])));
-            const unsigned c = u[0] + nx * u[1] + nxy * u[2];
+            const unsigned c = min(u[0] + nx * u[1] + nxy * u[2], kNoCell - 1u);  // (kWide: any number)
             const bool in = __float_as_int(q[k].w) >= 0;
             area[i] = in ? c : kNoCell;
             if (in) word[hash ? __umulhi(c * mult, nslots) : c] = static_cast<unsigned short>(i);
@@ -384,9 +462,9 @@ __device__ __noinline__ void far_cells(const float4* stg, int n, const PassGrid*
     }
 }
 
-// kDirect and kHash: the cells this thread's points (t0, t0 + T, ...) stand for.  The area holds
-// the points' cell numbers and nslots 16-bit words behind them.  kRare: of a far box (in a
-// function of its own: code beside the loops below costs every pass).
+// kDirect, kHash and kWide: the cells this thread's points (t0, t0 + T, ...) stand for.  The
+// area holds the points' cell numbers and nslots 16-bit words behind them.  kRare: of a far
+// box or kWide (in a function of its own: code beside the loops below costs every pass).
 template <bool SM, int T, bool kRare>
 __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const PassGrid* pg, int t0) {
     // Points of a group: more of them cost padding in the last group and code (16 / 8 /
@@ -395,11 +473,14 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
     static_assert(kSmallMax <= 64 * kST, "one bit per point of a thread: n <= 64 T");
     uint32_t* const area = pass_area<SM>();
     unsigned short* const word = reinterpret_cast<unsigned short*>(area + n);
-    const bool hash = pg->mode == kHash;
+    const bool hash = pg->mode != kDirect;
     const unsigned nslots = pg->nslots;
     const unsigned mult = 0x9E3779B1u;
     SmallSmem& sm = smem();
-    if (threadIdx.x == 0) sm.nopen[0] = 0;
+    if (threadIdx.x == 0) {
+        sm.nopen[0] = 0;
+        if (kRare) sm.ntwin = 0;
+    }
     // group(i0, all): the points i0, i0 + T, ... of which `all`, or those below n, are there.
     // A thread's loops run over whole groups, free of range checks, and one more
     auto each = [&](auto&& group) {
@@ -411,7 +492,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
 #pragma unroll 1
         for (; i0 < n; i0 += kIn * T) group(i0, std::false_type{});
     };
-    if constexpr (kRare) {
+    if (kRare && pg->far) {
         far_cells<SM, T>(stg, n, pg, word, mult, t0);
     } else {
         const CellMap cell(pg->bg);
@@ -432,6 +513,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
 #pragma unroll
             for (int k = 0; k < kIn; ++k) {
                 const int i = i0 + k * T;
+                if (kRare) c[k] = min(c[k], kNoCell - 1u);  // (kWide: any number)
                 if (__float_as_int(q[k].w) < 0) c[k] = kNoCell;  // taken
                 if (all.value || i < n) {
                     area[i] = c[k];
@@ -456,10 +538,10 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
     }
     // a slot's last writer stands for its cell; the points of the other cells that
     // share the slot are listed (a bit per point, then their indices)
-    unsigned long long left = 0;
+    unsigned long long left = 0, same = 0;
     int k0 = 0;
     each([&](int i0, auto all) {
-        unsigned c[kIn], w[kIn], bits = 0u;
+        unsigned c[kIn], w[kIn], bits = 0u, eq = 0u;
 #pragma unroll
         for (int k = 0; k < kIn; ++k) c[k] = (all.value || i0 + k * T < n) ? area[i0 + k * T] : kNoCell;
 #pragma unroll
@@ -470,18 +552,22 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
             if (c[k] != kNoCell) {
                 won += (w[k] == static_cast<unsigned>(i0 + k * T)) ? 1u : 0u;
                 bits |= (other != c[k]) ? (1u << k) : 0u;
+                if (kRare) eq |= (other == c[k] && w[k] != static_cast<unsigned>(i0 + k * T)) ? (1u << k) : 0u;
             }
         }
         left |= static_cast<unsigned long long>(bits) << k0;
+        if (kRare) same |= static_cast<unsigned long long>(eq) << k0;
         k0 += kIn;
     });
+    const bool wide = kRare && pg->mode == kWide;
+    if (wide) wide_check<SM>(stg, pg, word, nslots, mult, same, t0, T, nullptr);
     unsigned short* const list = reinterpret_cast<unsigned short*>(dyn + kListOff);
     append_open(left, t0, T, list, kOpenA);
     __syncthreads();
     int c = sm.nopen[0];
     unsigned more;
     if (c <= kOpenA) {
-        more = settle_open(area, word, nslots, c, list, kOpenA, list + kOpenA, kSelMax - kOpenA);
+        more = settle_open<SM, kRare>(stg, pg, word, nslots, c, list, kOpenA, list + kOpenA, kSelMax - kOpenA);
     } else {
         // too many for the list (levels near 32,768 points in about as many cells):
         // half of the words, which are done with, take it
@@ -493,9 +579,16 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
         __syncthreads();
         c = sm.nopen[0];
         if (c > half) return kManyOpen;
-        more = settle_open(area, word, half, c, word + half, half, list, kSelMax);
+        more = settle_open<SM, kRare>(stg, pg, word, half, c, word + half, half, list, kSelMax);
     }
-    return (more != kManyOpen) ? won + more : kManyOpen;
+    if (more == kManyOpen) return kManyOpen;
+    won += more;
+    if (wide) {
+        const unsigned own = count_twins();
+        if (own == kManyOpen) return kManyOpen;
+        won += own;
+    }
+    return won;
 }
 
 // kHash where many cells share slots: rounds with other hashes until few points
@@ -547,12 +640,13 @@ __device__ __noinline__ unsigned count_open(int n, const PassGrid* pg, int t0) {
     return won;
 }
 
-// kIndex: the number of points whose voxel was new; nslots words, more than points.
+// kIndex: the number of points whose voxel was new; more words than points.
 template <bool SM, int T>
 __device__ __noinline__ unsigned count_index(const float4* src, int n, const PassGrid* pg, int t0) {
     uint32_t* const area = pass_area<SM>();
     const Grid& G = pg->bg.g;
-    const unsigned nslots = pg->nslots;
+    constexpr unsigned kArea = static_cast<unsigned>((SM ? kTabBytes : kPtsBytes + kTabBytes) / 4);
+    const unsigned nslots = min(static_cast<unsigned>(2 * n + 64), kArea);
     const int tid = threadIdx.x;
     for (unsigned k = tid; k < nslots; k += kST) area[k] = 0u;
     __syncthreads();
@@ -591,16 +685,22 @@ __device__ __noinline__ unsigned count_index(const float4* src, int n, const Pas
     return fresh;
 }
 
-// The voxels of a size that this thread's points (t0, t0 + T, ...) count.
+// The voxels of a size that this thread's points (t0, t0 + T, ...) count.  (On one CTA,
+// whose few points hardly repay the code, far boxes and kWide take the general
+// ways: with them 1,000 points took 48.3 us, without 47.2.)
 template <bool SM, int T>
 __device__ __forceinline__ unsigned count_pass(const float4* stg, int n, const PassGrid* pg, int t0) {
-    if (pg->mode == kDirect || pg->mode == kHash) {
-        const unsigned won = (T == kST && pg->far) ? count_cells<SM, kST, true>(stg, n, pg, t0)
-                                                   : count_cells<SM, T, false>(stg, n, pg, t0);
-        return (won != kManyOpen) ? won : count_open<SM, T>(n, pg, t0);
+    constexpr bool kCluster = T == kST;
+    const int mode = pg->mode;
+    if (mode == kSkip) return 0u;
+    if (mode < kWide || (kCluster && mode == kWide)) {
+        const unsigned won = (kCluster && (mode == kWide || pg->far)) ? count_cells<SM, kST, true>(stg, n, pg, t0)
+                                                                      : count_cells<SM, T, false>(stg, n, pg, t0);
+        if (won != kManyOpen) return won;
+        if (mode != kWide) return count_open<SM, T>(n, pg, t0);
+        __syncthreads();  // (the count's area is filled anew)
     }
-    if (pg->mode == kIndex) return count_index<SM, T>(stg, n, pg, t0);
-    return 0u;
+    return count_index<SM, T>(stg, n, pg, t0);
 }
 
 // The grids of up to ten sizes over the level's box into sm.pg[first ...], how
@@ -631,14 +731,12 @@ __device__ __noinline__ void set_grids(int first, int sizes, float sv, const flo
         if (ax == 0) {
             const bool all_ok = (okm & 7u) == 7u, fast = all_ok && nx && ny && nz;
             const unsigned long long cells = static_cast<unsigned long long>(nx) * ny * nz;
-            // 16-bit words behind the cell numbers; for the load, 4 a point of kHash
+            // 16-bit words behind the cell numbers; for the load, 4 a point of kHash and kWide
             const unsigned words = 2u * (area_words - static_cast<unsigned>(n));
-            const bool direct = fast && cells <= words, hashed = fast && cells < kNoCell;
+            const bool direct = fast && cells <= words;
             g.sv = sv;
-            g.mode = direct ? kDirect : (hashed ? kHash : (all_ok ? kIndex : kSkip));
-            g.nslots = direct ? static_cast<unsigned>(cells)
-                              : (hashed ? min(words, 4u * static_cast<unsigned>(n))
-                                        : min(static_cast<unsigned>(2 * n + 64), area_words));
+            g.mode = !fast ? (all_ok ? kIndex : kSkip) : (direct ? kDirect : (cells < kNoCell ? kHash : kWide));
+            g.nslots = direct ? static_cast<unsigned>(cells) : min(words, 4u * static_cast<unsigned>(n));
             g.far = isinf(vmax) ? 1 : 0;
             g.bg.amb = __fmul_rn(vmax, kNear);
             g.bg.nx = nx;
