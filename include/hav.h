@@ -202,7 +202,11 @@ typedef struct {
                                 thread-block clusters, one cluster of 8 or 16 SMs
                                 per segment, each SM counting another size of the
                                 search (same results; settled steps as in the
-                                grid kernel; same conditions as solo_points) */
+                                grid kernel; same conditions as solo_points).
+                                A single cloud's level above 30,000 points with a
+                                budget of 3/8 of them (7/8 with several layers) or
+                                more stays on the grid-wide kernel where
+                                cluster_ctas is 0 and a size is searched */
     int32_t solo_points;     /* levels whose every segment has at most this many
                                 points (0..4096; 0: none; default 4096) run on
                                 single CTAs, one per segment, its points and

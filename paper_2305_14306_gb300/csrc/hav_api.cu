@@ -345,7 +345,18 @@ hav_status hav_sample_batched(hav_ctx* ctx, const float* points, const int64_t* 
                                             : seg_m[static_cast<int64_t>(j - 1) * num_segments + s];
                 if (nj > mx) mx = nj;
             }
-            const bool clusters = small_ok && ctx->small_points > 0 && mx <= ctx->small_points;
+            // One large cloud and a large budget: the grid kernel (cluster_ctas 0).  Each
+            // CTA counts all of the level's points, and above kClusterAlone points the
+            // words of its shared memory are hardly more than the voxels of the sizes
+            // near such a budget.  (GB300, 32,768 points, mean over rooms, boxes and
+            // scans by time on a cluster / on the grid: one layer to 3/4 122 / 101 us,
+            // to 9/10 119 / 104, to 3/10 102 / 96; two layers to 97/100 171 / 140, to
+            // 3/4 146 / 141, to 3/10 139 / 149.)
+            const int64_t mj = seg_m[static_cast<int64_t>(j) * num_segments];
+            const bool large = num_segments == 1 && ctx->cluster_ctas == 0 && mx > havk::kClusterAlone &&
+                               params->t_max > 0 && !(params->fixed_s > 0.0f) &&
+                               8 * mj >= (params->layers == 1 ? 3 : 7) * mx;
+            const bool clusters = small_ok && ctx->small_points > 0 && mx <= ctx->small_points && !large;
             const bool solo = small_ok && ctx->solo_points > 0 && mx <= ctx->solo_points &&
                               (ctx->small_points == 0 || num_segments > ctx->small_nc || mx <= havk::kSoloAlone);
             if (j0 == num_levels && (clusters || solo)) j0 = j;

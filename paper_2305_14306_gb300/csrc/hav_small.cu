@@ -98,7 +98,7 @@ __host__ __device__ constexpr int qlog2() {
 //            stand for do so (equal numbers read the same word): they are
 //            collected with their keys, and their distinct keys added.  In a
 //            scan hardly two cells share a number.  (16 CTAs, a LiDAR scan of
-//            24,000 points to 97 of 100, one layer: 217 us by kIndex, 101 so; a
+//            24,000 points to 97 of 100, one layer: 213 us by kIndex, 113 so; a
 //            pass 30 us, 17 to 21 by kHash.)
 //   kIndex   (a cell index that may be out of range, more points with a shared
 //            number than are collected, or 2^32 cells on one CTA) open addressing
