@@ -48,14 +48,14 @@ __global__ void __launch_bounds__(kFpsThreads, 1)
     const int a = blockIdx.x * chunk;
     const int b = min(n, a + chunk);
     for (int i = a + tid; i < b; i += kFpsThreads) {
-        if constexpr (kResident) res[i - a] = make_float4(pts[3 * i], pts[3 * i + 1], pts[3 * i + 2], INFINITY);
+        if constexpr (kResident) res[i - a] = make_float4(pts[3ll * i], pts[3ll * i + 1], pts[3ll * i + 2], INFINITY);
         else dist_g[i] = INFINITY;
     }
     int last = 0;
     if (blockIdx.x == 0 && tid == 0) out[0] = 0;
     __syncthreads();
     for (int j = 1; j < m; ++j) {
-        const float qx = pts[3 * last], qy = pts[3 * last + 1], qz = pts[3 * last + 2];
+        const float qx = pts[3ll * last], qy = pts[3ll * last + 1], qz = pts[3ll * last + 2];
         unsigned long long best = 0ull;
         for (int i = a + tid; i < b; i += kFpsThreads) {
             float px, py, pz, di;
@@ -75,9 +75,9 @@ __global__ void __launch_bounds__(kFpsThreads, 1)
             }
             if (di < 0.0f) continue;
             if constexpr (!kResident) {
-                px = pts[3 * i];
-                py = pts[3 * i + 1];
-                pz = pts[3 * i + 2];
+                px = pts[3ll * i];
+                py = pts[3ll * i + 1];
+                pz = pts[3ll * i + 2];
             }
             const float dx = __fsub_rn(px, qx);
             const float dy = __fsub_rn(py, qy);

@@ -529,7 +529,7 @@ __device__ __forceinline__ void for_points(const float* points, int a, int b, F&
         float p[4][3];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float* q = points + 3 * min(i0 + k * kThreads, b - 1);
+            const float* q = points + 3ll * min(i0 + k * kThreads, b - 1);  // (beyond 2^31 floats from 715,827,883 points on)
 #pragma unroll
             for (int a3 = 0; a3 < 3; ++a3) p[k][a3] = __ldg(q + a3);
         }
