@@ -695,7 +695,7 @@ __device__ __forceinline__ void cell_axes(unsigned c, const ItemGrid& g, unsigne
 // candidate's table; whether it was not set before, and its slot (neighbouring
 // cells in different ones).
 __device__ __forceinline__ bool set_bit(unsigned long long* T, int cap_log2, unsigned cell, long long* slot) {
-    *slot = cell & ((1u << cap_log2) - 1u);
+    *slot = cell & (0xffffffffu >> (32 - cap_log2));  // (up to 2^32 slots)
     const unsigned bit = static_cast<unsigned>(static_cast<unsigned long long>(cell) >> cap_log2);
     const unsigned m = 1u << (bit & 31u);
     unsigned* const wd = reinterpret_cast<unsigned*>(T + *slot) + (bit >> 5);
@@ -756,7 +756,7 @@ __device__ __noinline__ int pass_keys(const float4* ord, const ItemGrid* ig, int
 // find_or_insert with a compare-and-swap for every probe (one round trip where
 // the first slot is empty or holds the key); bit 62 of the result: fresh.
 __device__ __noinline__ long long insert_key(unsigned long long* T, int cap_log2, unsigned long long key) {
-    const unsigned mask = (1u << cap_log2) - 1u;
+    const unsigned mask = 0xffffffffu >> (32 - cap_log2);
     unsigned slot = static_cast<unsigned>(slot_mix(key) >> (64 - cap_log2));
 #pragma unroll 1
     for (unsigned probe = 0; probe <= mask; ++probe) {
@@ -2091,8 +2091,8 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 if (tid < S && (st.flags[tid] & F_ACTIVE) && st.kstar[tid] > st.ml[tid]) {
                     c = static_cast<int>(ld_volatile(reinterpret_cast<const int*>(&ls[tid].cand)));
                     // only the first C/2 were stored (the rest reported a full table)
-                    const int cmax = 1 << (st.cap_log2[tid] - 1);
-                    if (c > cmax) c = cmax;
+                    const long long cmax = 1ll << (st.cap_log2[tid] - 1);
+                    if (c > cmax) c = static_cast<int>(cmax);
                 }
                 int ctot;
                 const int cpre = block_excl_scan<int>(tid < S ? c : 0, &ctot, st.scan_i);

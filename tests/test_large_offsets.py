@@ -1,6 +1,6 @@
-"""Offsets of points beyond 2^31 floats (clouds of more than 715,827,882 points,
+"""Addresses of large calls: points beyond 2^31 floats (clouds of more than 715,827,882 points,
 which a context may be created for): the grid kernel's read of the input
-points, built for the host."""
+points, built for the host, and the slots of its tables."""
 import ctypes as C
 
 import pytest
@@ -42,3 +42,48 @@ def test_input_points(tmp_path, first):
         want = {4 * (3 * i + a) for i in range(first + tid, first + 3001, 512) for a in range(3)}
         last = {4 * (3 * (first + 3000) + a) for a in range(3)}  # (read in place of points behind the last)
         assert want <= seen <= want | last
+
+
+TABLE = r"""
+static unsigned long long touched;
+static unsigned atomicAnd(unsigned* p, unsigned) { touched = reinterpret_cast<uintptr_t>(p); return ~0u; }
+static unsigned long long atomicCAS(unsigned long long* p, unsigned long long e, unsigned long long) {
+    touched = reinterpret_cast<uintptr_t>(p);
+    return e;
+}
+constexpr unsigned long long kEmptyKey = ~0ull;
+%s
+extern "C" long long bit_of(int cap, unsigned cell, unsigned long long* at) {
+    long long slot = -1;
+    const bool fresh = set_bit(reinterpret_cast<unsigned long long*>(uintptr_t(1) << 20), cap, cell, &slot);
+    *at = touched - (1 << 20);
+    return fresh ? slot : -2;
+}
+extern "C" long long key_of(int cap, unsigned long long key, unsigned long long* at, unsigned long long* hash) {
+    const long long r = insert_key(reinterpret_cast<unsigned long long*>(uintptr_t(1) << 20), cap, key);
+    *at = touched - (1 << 20);
+    *hash = slot_mix(key);
+    return r & ~(1ll << 62);
+}
+"""
+
+
+# tables of the smallest capacity to 2^32 slots (an eighth full with 2^29 points)
+@pytest.mark.parametrize("cap", [6, 7, 17, 30, 31, 32])
+def test_table_slots(tmp_path, cap):
+    mix = H.passage("hav_device.cuh", "__device__ __forceinline__ unsigned long long slot_mix(",
+                    "// Slot hash of the block-local sets")
+    bit = H.passage("hav_sampler.cu", "__device__ __forceinline__ bool set_bit(", "// The units of a tile whose cells or keys")
+    key = H.passage("hav_sampler.cu", "__device__ __noinline__ long long insert_key(",
+                    "// A bisection pass over this block's work items")
+    lib = H.compile_host(tmp_path, TABLE % (mix + bit + key))
+    lib.bit_of.restype = lib.key_of.restype = C.c_longlong
+    at, h = C.c_ulonglong(), C.c_ulonglong()
+    top = min(64 << cap, 2**32 - 1)
+    for cell in [0, 1, 63, 64, top - 1, top // 2, top // 3, (1 << min(cap, 31)) - 1]:
+        slot = lib.bit_of(cap, C.c_uint(cell), C.byref(at))
+        assert slot == cell % 2**cap
+        assert at.value == 8 * slot + 4 * ((cell >> cap) // 32)
+    for k in (0, 5, 12345678901234567, 2**63 - 1):
+        slot = lib.key_of(cap, C.c_ulonglong(k), C.byref(at), C.byref(h))
+        assert slot == h.value >> (64 - cap) and at.value == 8 * slot
