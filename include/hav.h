@@ -351,11 +351,12 @@ hav_status hav_count(hav_ctx* ctx, const float* points, int64_t n, float s,
  * n*3 floats; out_idx: device, m int32 in selection order.  0 <= m <= n <=
  * the context's max_points.  One launch: up to 196,608 points one cluster of
  * 16 CTAs (or 8: up to 98,304) that holds the points and their distances in
- * its shared memory and picks many points per cluster barrier (up to
- * 32,768 points and some 20 to 60 picks one per barrier); above that, and for up
- * to some 60 to 140 picks from 32,769 points on, a cooperative grid with one grid barrier per selected point (each block's
- * share of the points and their distances held in its shared memory where 16
- * bytes a point fit, about 1.9 M points on 152 SMs); asynchronous on
+ * its shared memory and picks many points per cluster barrier (a few picks,
+ * some 20 to 60, of up to 32,768 points one per barrier); above that, and for
+ * up to some 60 to 140 picks from 32,769 points on, a cooperative grid with one
+ * grid barrier per selected point (each block's share of the points and their
+ * distances held in its shared memory where 16 bytes a point fit, about 1.9 M
+ * points on 152 SMs); asynchronous on
  * `stream`; a grid barrier timeout is read with hav_status_get. */
 hav_status hav_fps(hav_ctx* ctx, const float* points, int64_t n, int64_t m, int32_t* out_idx,
                    hav_stream stream);

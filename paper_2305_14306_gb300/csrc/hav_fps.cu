@@ -512,7 +512,10 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kFpsBatchThreads, 1)
         __syncthreads();
         k = sm.npick;
         j += k;
-        if (total < 40) drop = fminf(0.9f, drop * 1.25f);
+        // (a long list lowers it at every look, which suits a run of tied distances,
+        // to 0 in the end; from there, and from far below what distinct distances
+        // need, it has to come back)
+        if (total < 40) drop = fminf(0.9f, drop * (drop < 1e-2f ? 2.0f : 1.25f) + 1e-7f);
         else if (total > 80) drop *= 0.8f;
         thr = static_cast<unsigned long long>(__float_as_uint(__fmul_rn(sm.last, 1.0f - drop))) << 32;
         have_over = false;

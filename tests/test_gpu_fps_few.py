@@ -60,3 +60,15 @@ def test_forms(hv, ctx, oracle_mod, form):
            "same": lambda: np.ones((8000, 3)),
            "not finite": lambda: np.where(rng.random((8000, 1)) < 0.002, np.array([[np.nan, 1, np.inf]]), box)}[form]()
     check(hv, ctx, oracle_mod, pts, line(8000) - 1)
+
+
+# tied distances first, distinct ones after them (and mixed): the threshold's distance comes back from 0
+@pytest.mark.parametrize("form", ["half rounded", "lattice, then a box", "a fine box in a lattice"])
+def test_ties_and_distinct_distances(hv, ctx, oracle_mod, form):
+    rng = np.random.default_rng(5)
+    box = scenes.uniform_box(9000, 6)
+    grid = np.stack(np.meshgrid(*[np.arange(16)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    pts = {"half rounded": lambda: rng.permutation(np.concatenate([np.rint(box[:4000]), box[4000:8000]])),
+           "lattice, then a box": lambda: np.concatenate([grid * 30.0, box[:4000]]),
+           "a fine box in a lattice": lambda: np.concatenate([grid * 1.0, box[:4000] * 0.2])}[form]()
+    check(hv, ctx, oracle_mod, pts, 2500)
