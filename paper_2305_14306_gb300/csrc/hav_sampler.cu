@@ -661,7 +661,8 @@ __device__ __noinline__ void item_grids(int S, unsigned nb, int w0, int li0, int
         g.nslots = cells <= words ? static_cast<unsigned>(cells) : words;
         g.mode = !all_ok ? kCountNone
                          : (!fast || cells >= kNoCell ? kCountKeys : (cells <= words ? kCountDirect : kCountHash));
-        const bool bits = scells < kNoCell && scells <= (64ull << st.cap_log2[s]);
+        // (no cells: the box is too long along an axis, or the size is not representable)
+        const bool bits = scells != 0ull && scells < kNoCell && scells <= (64ull << st.cap_log2[s]);
         g.snx = bits ? sx : 0u;
         g.snxy = sx * sy;
         // (two candidates and more share the tables' room)
@@ -2100,7 +2101,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 if (tid == 0) st.cprefix[S] = ctot;
                 __syncthreads();
                 // a warp per candidate, the segment's candidates split over its lanes
-                // (one thread each took 27 us for the 836 of 856,000 voxels, half of
+                // (one thread each took 66 us for the 836 of 856,000 voxels, half of
                 // the phase's time in a usual layer)
 #pragma unroll 1
                 for (int w = (tid >> 5) * static_cast<int>(nb) + static_cast<int>(blockIdx.x); w < ctot;

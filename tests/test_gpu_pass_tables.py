@@ -55,3 +55,41 @@ def test_outliers_in_one_item(hv, n, wide, search, depth, table_log2):
                 assert np.array_equal(out, res[0]), m
     finally:
         ctx.close()
+
+
+# a box of 2^21 cells and more along one axis and few along the others (keys, never
+# bits): the call and an ordinary one after it on the same tables
+@pytest.mark.parametrize("depth", [[NEVER, NEVER, NEVER], *DEPTHS.values()])
+@pytest.mark.parametrize("search", ["bisect", "guided"])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_long_axis(hv, axis, search, depth):
+    import oracle
+    rng = np.random.default_rng(axis)
+    long = rng.uniform(0, 1, (20000, 3)) * np.array([4e-3, 4e-3, 3e-3])
+    long = long[rng.integers(0, 9000, 20000)]  # (repeats: never as many voxels as points)
+    long[:, axis] = rng.uniform(0, 1e-3, 20000)[rng.integers(0, 9000, 20000)]
+    long[77, axis], long[15000, axis] = 3000.0, 900.0
+    box = rng.uniform(-5, 5, (30000, 3))
+    clouds = [(np.ascontiguousarray(c, dtype=np.float32), m) for c, m in ((long, [19000]), (box, [20000, 4000]))]
+    kw = dict(search=search)
+    p = hv.params(**kw)
+    ctx = hv.Context(1 << 17, 1)
+    try:
+        ctx.set_tuning(small_points=0, solo_points=0, spec_points=depth)
+        for pts, m in (clouds[1], clouds[0], clouds[1], clouds[0], clouds[1]):
+            outs = hv.hav_sample_levels(ctx, torch.from_numpy(pts).cuda(), m, p)
+            status = hv.hav_status_get(ctx, 1)[0]
+            try:
+                (res, tro), = G.oracle_many([pts], [m], kw)
+            except oracle.OracleError as e:
+                assert status == e.status
+                continue
+            assert status == 0
+            tr = hv.hav_trace_get(ctx, len(m) * p.layers)
+            for j in range(len(m)):
+                for l in range(p.layers):
+                    why = G.traces_equal(tr[j * p.layers + l], tro[j][l])
+                    assert why is None, (j, l, why)
+                assert np.array_equal(outs[j].cpu().numpy(), res[j]), j
+    finally:
+        ctx.close()
