@@ -360,7 +360,9 @@ __device__ __forceinline__ unsigned bucket_of(const float p[3], const float mn[3
 // than 1e-5, so widening the ends by 0.01 cells yields every cell a point of
 // the voxel can fall in (outside [0, 16] the clamp to the end cells decides).
 // Morton order is monotone in each cell coordinate, so those cells lie
-// between the codes of the two corner cells.  k[a] = RN(16 / e_a), 0 if e_a = 0.
+// between the codes of the two corner cells.  k[a] = RN(16 / e_a), 0 if e_a = 0;
+// where it overflows (extents below 5e-38) nothing is owned (scales_ok).
+__device__ __forceinline__ bool scales_ok(const float k[3]) { return isfinite(k[0]) && isfinite(k[1]) && isfinite(k[2]); }
 __device__ __forceinline__ bool voxel_owned(unsigned long long key, const Grid& g, const float mn[3],
                                             const float k[3], int own_lo, int own_hi) {
     unsigned c0[3], c1[3];
@@ -405,7 +407,7 @@ __device__ void own_cells(const uint32_t* hb, int ia, int ib, unsigned end, cons
     }
     st.own_lo[li] = c_lo;
     st.own_hi[li] = lo - 1;
-    st.own_on[li] = (c_lo <= lo - 1) ? 1 : 0;
+    st.own_on[li] = (c_lo <= lo - 1 && scales_ok(k)) ? 1 : 0;
     for (int a3 = 0; a3 < 3; ++a3) {
         st.own_mn[li][a3] = mn[a3];
         st.own_k[li][a3] = k[a3];
@@ -1286,7 +1288,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 const int hi = (ib == se || cell(ib) > cl) ? cl : cl - 1;
                 st.own_lo[li] = lo;
                 st.own_hi[li] = hi;
-                st.own_on[li] = (lo <= hi) ? 1 : 0;
+                st.own_on[li] = (lo <= hi && scales_ok(k3)) ? 1 : 0;
                 for (int a3 = 0; a3 < 3; ++a3) {
                     st.own_mn[li][a3] = mn3[a3];
                     st.own_k[li][a3] = k3[a3];
@@ -1309,7 +1311,7 @@ __global__ void __launch_bounds__(kThreads, 1) hav_chain_kernel(const __grid_con
                 const int hi = (ib == NL || cell(ib) > cl) ? cl : cl - 1;
                 st.own_lo[li] = lo;
                 st.own_hi[li] = hi;
-                st.own_on[li] = (lo <= hi) ? 1 : 0;
+                st.own_on[li] = (lo <= hi && scales_ok(st.b0_k)) ? 1 : 0;
                 for (int a3 = 0; a3 < 3; ++a3) {
                     st.own_mn[li][a3] = st.b0_mn[a3];
                     st.own_k[li][a3] = st.b0_k[a3];

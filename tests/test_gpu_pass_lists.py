@@ -50,3 +50,32 @@ def test_owned_beside_undecided(hv, cloud, m, depth):
                     assert why is None, (j, l, why)
     finally:
         ctx.close()
+
+
+# extents so small that the sorting cells' scale 16 / extent overflows (or hardly does not): nothing is owned
+@pytest.mark.parametrize("extent", [2e-38, 4.6e-38, 6e-38])
+@pytest.mark.parametrize("sizes", [[140_000], [30_000, 60_000, 440_000]])
+def test_sorted_tiny_extents(hv, sizes, extent):
+    rng = np.random.default_rng(7)
+    clouds = [np.ascontiguousarray(rng.uniform(0, extent, (n, 3)), dtype=np.float32) for n in sizes[:2]]
+    clouds += [scenes.uniform_box(n, n) for n in sizes[2:]]
+    levels = [[len(c) // 3, len(c) // 10] for c in clouds]
+    want = G.oracle_many(clouds, levels)
+    pts, offs = scenes.concat(clouds)
+    m = np.array(levels, dtype=np.int64).T
+    p = hv.params()
+    ctx = hv.Context(int(offs[-1]), len(clouds))
+    try:
+        ctx.set_tuning(small_points=0, solo_points=0)
+        outs = [o.cpu().numpy() for o in hv.hav_sample_batched(ctx, torch.from_numpy(pts).cuda(), offs, m, p)]
+        assert hv.hav_status_get(ctx, len(clouds))[0] == 0
+        tr = hv.hav_trace_get(ctx, m.size * p.layers)
+    finally:
+        ctx.close()
+    for s, (res, tro) in enumerate(want):
+        for j in range(2):
+            for l in range(p.layers):
+                why = G.traces_equal(tr[(j * len(clouds) + s) * p.layers + l], tro[j][l])
+                assert why is None, (s, j, l, why)
+            a = int(m[j, :s].sum())
+            assert np.array_equal(outs[j][a:a + m[j, s]], res[j]), (s, j)
