@@ -36,9 +36,11 @@ constexpr int kMaxCand = (1 << kMaxSpecDepth) - 1;  // candidate sizes per pass 
 // set (p - 1) % 3 while it waits, ready for pass p + 2.
 constexpr int kTableSets = 3;
 // default level sizes (points) up to which a pass evaluates 4, 3 or 2 steps
-// ahead (measured on GB300: 15 candidates per pass never paid off; with the
-// coarse steps settled without a pass, the passes left are near the target,
-// where 7 candidates pay up to about 4k points and 3 up to 64k)
+// ahead.  Measured on GB300, one level on the grid kernel, mean of boxes, rooms and
+// scans to a quarter and a sixteenth, with one / two / three steps a pass (15
+// candidates never paid off): 2,048 points 164 / 136 / 134 us, 4,096 156 / 134 /
+// 128, 8,192 149 / 129 / 130, 32,768 176 / 155 / 159, 65,536 149 / 138 / 154,
+// 98,304 164 / 156 / 177, 131,072 191 / 189 / 214, 262,144 206 / 235 / 235.
 constexpr int64_t kSpecN4 = 0;
 constexpr int64_t kSpecN3 = 4096;
 constexpr int64_t kSpecN2 = 65536;

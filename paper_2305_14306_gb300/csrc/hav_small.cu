@@ -27,10 +27,10 @@
 // -> 63.6 us, LiDAR chain 20,876 -> 16,384 -> 4,096 -> 1,024 -> 512 364 -> 289
 // us, 64 clouds of 1,000-4,000 points, two levels, 144 -> 105 us.
 //
-// The selection at s* is spread by voxel: every CTA goes through all points
-// and keeps those whose voxel hashes to it, so that the table of a voxel's
-// closest point is in the CTA's own shared memory too.  Only the cut-off
-// histograms, the boundary bin's candidates and the counts of kept points
+// The selection at s* is spread by voxel: every CTA hands the points of its share
+// to the CTAs that their voxels hash to, as records that those fetch, so that the
+// table of a voxel's closest point is in a CTA's own shared memory too.  Only the
+// records, the cut-off histograms, the boundary bin's candidates and the counts of kept points
 // cross the cluster, and the taken marks through the staged points in global
 // memory (a level of at most kPtsSmem points also has a copy in shared memory,
 // re-marked at the start of a layer; Q = 1 works on that copy alone).
@@ -76,7 +76,7 @@ static_assert(16 * (2 * kPtsSmem / 8) + 16 * (kPtsSmem / 8) <= kTabBytes, "selec
 
 template <int Q>
 __host__ __device__ constexpr int qlog2() {
-    return Q == 16 ? 4 : (Q == 8 ? 3 : (Q == 4 ? 2 : (Q == 2 ? 1 : 0)));
+    return Q == 16 ? 4 : (Q == 8 ? 3 : 0);
 }
 
 // How a pass counts distinct voxels among the cells the bounding box spans.
@@ -297,8 +297,8 @@ __device__ __forceinline__ uint32_t* pass_area() {
     return reinterpret_cast<uint32_t*>(SM ? dyn + kPtsBytes : dyn);
 }
 
-// The counting functions are not inlined: each gets the whole register budget
-// of a thread (64) instead of what the kernel around it leaves.
+// The counting functions are not inlined: their loops get the registers of a
+// thread (128) that the kernel around them does not hold across the call.
 
 // The points t0 + b T of a thread's set bits b to the list, of which the first
 // `room` are kept (whole warps; one atomic a warp).
