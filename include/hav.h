@@ -206,7 +206,8 @@ typedef struct {
                                 A single cloud's level above 30,000 points with a
                                 budget of 3/8 of them (7/8 with several layers) or
                                 more stays on the grid-wide kernel where
-                                cluster_ctas is 0 and a size is searched */
+                                cluster_ctas is 0, a size is searched and the
+                                context has at least 76 blocks */
     int32_t solo_points;     /* levels whose every segment has at most this many
                                 points (0..4096; 0: none; default 4096) run on
                                 single CTAs, one per segment, its points and

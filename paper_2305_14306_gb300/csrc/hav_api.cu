@@ -351,10 +351,11 @@ hav_status hav_sample_batched(hav_ctx* ctx, const float* points, const int64_t* 
             // near such a budget.  (GB300, 32,768 points, mean over rooms, boxes and
             // scans by time on a cluster / on the grid: one layer to 3/4 122 / 101 us,
             // to 9/10 119 / 104, to 3/10 102 / 96; two layers to 97/100 171 / 140, to
-            // 3/4 146 / 141, to 3/10 139 / 149.)
+            // 3/4 146 / 141, to 3/10 139 / 149.  With 100 / 76 / 48 of the 152 blocks the
+            // grid takes 105 / 109 / 128 us to 3/4, a cluster 117.)
             const int64_t mj = seg_m[static_cast<int64_t>(j) * num_segments];
             const bool large = num_segments == 1 && ctx->cluster_ctas == 0 && mx > havk::kClusterAlone &&
-                               params->t_max > 0 && !(params->fixed_s > 0.0f) &&
+                               plan->nblocks >= havk::kGridBlocks && params->t_max > 0 && !(params->fixed_s > 0.0f) &&
                                8 * mj >= (params->layers == 1 ? 3 : 7) * mx;
             const bool clusters = small_ok && ctx->small_points > 0 && mx <= ctx->small_points && !large;
             const bool solo = small_ok && ctx->solo_points > 0 && mx <= ctx->solo_points &&

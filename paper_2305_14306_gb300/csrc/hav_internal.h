@@ -47,6 +47,7 @@ constexpr int64_t kSpecN2 = 65536;
 constexpr int kChunkMin = 64;              // default smallest work item (points)
 constexpr int kSmallMax = 32768;           // largest level the cluster kernel takes (points)
 constexpr int kClusterAlone = 30000;       // one cloud's largest level that a cluster takes whatever its budget
+constexpr int kGridBlocks = 76;            // blocks with which the grid kernel is the faster one above it
 constexpr int kLocalItems = 8;             // work items one block can own in a level
 // Pass shapes of the grid kernel (template instantiations): points each thread
 // loads ahead in the selection, and probes of the global tables it keeps in

@@ -14,7 +14,8 @@ A context's knobs (``hav_tuning`` in include/hav.h) that the tuner searches:
   in flight, one instantiation of the grid kernel each (the block
   shape itself is fixed: one 512-thread block per SM);
 * ``small_points`` -- the level size up to which levels run on thread-block
-  clusters (0: never).
+  clusters (0: never; a single cloud's levels above 30,000 points with a large
+  budget stay on the grid kernel).
 
 The number of blocks is left as it is.  No knob changes a result.  The tuner
 therefore times the caller's own workload under a short list of settings (a

@@ -24,7 +24,7 @@ def hv():
     return hav
 
 
-# (points, budget, layers, extra parameters, launches of the call and of one with 16-CTA clusters asked for)
+# (points, budget, layers, extra parameters, launches of the call, and of one with clusters asked for or few blocks)
 @pytest.mark.parametrize("n,m,layers,kw,launches", [
     (30000, [29000, 2100], 1, {}, (1, 1)),
     (30001, [11250, 2100], 1, {}, (1, 1)),
@@ -43,8 +43,8 @@ def test_budgets(hv, n, m, layers, kw, launches):
     dev = torch.from_numpy(pts).cuda()
     ctx = hv.Context(n, 1)
     try:
-        for ctas, count in zip((0, 16), launches):
-            ctx.set_tuning(cluster_ctas=ctas)
+        for ctas, blocks, count in ((0, 0, launches[0]), (0, 76, launches[0]), (0, 75, launches[1]), (16, 0, launches[1])):
+            ctx.set_tuning(cluster_ctas=ctas, nblocks=blocks)
             before = ctx.launches()
             outs = hv.hav_sample_levels(ctx, dev, m, p)
             assert hv.hav_status_get(ctx, 1)[0] == 0
