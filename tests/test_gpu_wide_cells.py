@@ -1,7 +1,7 @@
 """Searches at sizes where the box spans 2^32 cells and more (small-level
-kernels): cells whose table entries look alike, scans at nearly every point a
-voxel, outliers.  Indices and traces bit-identical to the oracle's on every
-engine."""
+kernels): cells whose numbers agree modulo 2^32 or whose table entries look
+alike, scans at nearly every point a voxel, outliers.  Indices and traces
+bit-identical to the oracle's on every engine."""
 import os
 import sys
 
@@ -99,6 +99,33 @@ def test_entries_alike(hv, ctx, cells, others, repeats):
     assert int(tro[0][0]["iters"]) == 20
     check(hv, ctx, pts, [cells + others], sigma=(0, 1))
     check(hv, ctx, pts, [(cells + others) // 2], search="guided")
+
+
+def twins(pairs, repeats, seed):
+    """A cube of side E = 2^16 - 1 with pairs of points (1, -2, 1) E / 2^16
+    apart.  At size E / 2^t, t >= 16, the box has 2^t + 1 cells an axis and the
+    two cells' numbers differ by ((2^t)^2) 2^(t - 16), a multiple of 2^32."""
+    rng = np.random.default_rng(seed)
+    side = float(2**16 - 1)
+    s = side / 2**16
+    a = rng.integers(8, 2**16 - 8, (pairs, 3)) * s + 0.5 * s
+    b = a + np.array([1, -2, 1]) * s
+    close = a[: pairs // 8] + np.array([0.2, 0, 0.1]) * s  # apart from some t = 18 on
+    corners = np.array([[0, 0, 0], [side, side, side]], dtype=np.float64)
+    # cells 2^32 - 1 at t = 16: (0, 65535, 0)
+    marked = np.tile([[0.25 * s, 65535.5 * s, 0.25 * s]], (3, 1))
+    pts = np.concatenate([corners, marked, close] + [a, b] * repeats)
+    return pts[rng.permutation(len(pts))]
+
+
+# cells whose numbers agree modulo 2^32: few, and more than are collected
+@pytest.mark.parametrize("pairs,repeats", [(3, 3), (200, 2), (900, 2), (1900, 1), (5000, 2), (15000, 1)])
+def test_twins(hv, ctx, pairs, repeats):
+    pts = twins(pairs, repeats, pairs)
+    tro = check(hv, ctx, pts, [len(pts)], layers=1)  # (never enough voxels: every size of the search)
+    assert int(tro[0][0]["iters"]) == 20
+    check(hv, ctx, pts, [2 * pairs + 3 + pairs // 16], sigma=(0, 1), layers=1)
+    check(hv, ctx, pts, [pairs + pairs // 2, pairs // 3], search="guided")
 
 
 @pytest.mark.parametrize("n,m", [(4096, 4000), (12000, 11900), (20000, 18000), (32768, 31000), (32768, 32700)])
