@@ -58,6 +58,7 @@ constexpr int kWarps = kST / 32;
 constexpr int kPtsSmem = 4096;   // levels of at most this many points have a copy in shared memory (64 KB)
 constexpr int kSelMax = 8192;    // slots of a CTA's part of the selection table at most (128 KB)
 constexpr int kMaxQ = 16;        // largest cluster
+constexpr long long kWideMin = 8192;  // points from which a launch may take the kernels built for kWide
 constexpr int kCutBits = 6;      // cut-off histogram over the top priority bits
 constexpr int kCutBins = 1 << kCutBits;
 constexpr int kOpenA = kSelMax / 8 * 7;  // undecided points of a pass that are listed (in later rounds, alternately the rest)
@@ -91,8 +92,8 @@ __host__ __device__ constexpr int qlog2() {
 //            write.  (A bitmap and a table of cell numbers, one shared-memory
 //            atomic per point, took 1.7 to 2.5 times as long: neighbouring
 //            points' atomics meet in one word.)
-//   kWide    (2^32 cells and more, on a cluster) kHash on the cell numbers modulo
-//            2^32.  A point that reads one of its own number compares the cells
+//   kWide    (2^32 cells and more, in the kernels built for it) kHash on the cell
+//            numbers modulo 2^32.  A point that reads one of its own number compares the cells
 //            themselves (wide_check), a look at the points that share a voxel.
 //            Where the cells differ, all points of the one that the word does not
 //            stand for do so (equal numbers read the same word): they are
@@ -101,9 +102,13 @@ __host__ __device__ constexpr int qlog2() {
 //            24,000 points to 97 of 100, one layer: 213 us by kIndex, 113 so; a
 //            pass 30 us, 17 to 21 by kHash.)
 //   kIndex   (a cell index that may be out of range, more points with a shared
-//            number than are collected, or 2^32 cells on one CTA) open addressing
+//            number than are collected, or 2^32 cells elsewhere) open addressing
 //            on (16 key bits, point index) with atomics, compared through the
 //            indexed point's key
+// kWide's code is in kernels of its own (template argument kW), taken for large
+// budgets (launch_small): in one kernel with the other ways it cost registers that
+// every pass then spilled (16,384 uniform points to 4,096, caches cold, 68.3 us
+// without it, 72.0 with it).
 enum : int { kSkip = 0, kDirect = 1, kHash = 2, kWide = 3, kIndex = 4 };
 
 // A pass's size, its grid over the level's box, and how a pass counts it.
@@ -370,12 +375,12 @@ __device__ __noinline__ unsigned count_twins() {
 // among themselves with other hashes (what a round leaves goes to `other`, and
 // to and fro), the last few by a warp.  In every thread kManyOpen where a round
 // leaves too many.
-template <bool SM, bool kRare>
+template <bool SM, bool kW>
 __device__ __noinline__ unsigned settle_open(const float4* stg, const PassGrid* pg, unsigned short* word, unsigned nslots,
                                              int c, unsigned short* list, int list_room, unsigned short* other,
                                              int other_room) {
     const uint32_t* const area = pass_area<SM>();
-    const bool wide = kRare && pg->mode == kWide;
+    const bool wide = kW && pg->mode == kWide;
     SmallSmem& sm = smem();
     unsigned mult = 0xB7A56463u, won = 0;
 #pragma unroll 1
@@ -398,10 +403,10 @@ __device__ __noinline__ unsigned settle_open(const float4* stg, const PassGrid* 
             } else if (area[w] != mine) {
                 const int pos = atomicAdd(&sm.nopen[round & 1], 1);
                 if (pos < other_room) other[pos] = static_cast<unsigned short>(i);
-            } else if (kRare) {
+            } else if (kW) {
                 same |= 1ull << b;
             }
-            if (kRare) ++b;
+            if (kW) ++b;
         }
         if (wide) wide_check<SM>(stg, pg, word, nslots, mult, same, threadIdx.x, kST, list);
         __syncthreads();
@@ -464,8 +469,8 @@ __device__ __noinline__ void far_cells(const float4* stg, int n, const PassGrid*
 
 // kDirect, kHash and kWide: the cells this thread's points (t0, t0 + T, ...) stand for.  The
 // area holds the points' cell numbers and nslots 16-bit words behind them.  kRare: of a far
-// box or kWide (in a function of its own: code beside the loops below costs every pass).
-template <bool SM, int T, bool kRare>
+// box, or (kW) kWide, in a function of its own: code beside the loops below costs every pass.
+template <bool SM, int T, bool kRare, bool kW>
 __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const PassGrid* pg, int t0) {
     // Points of a group: more of them cost padding in the last group and code (16 / 8 /
     // 4 / 2 / 1 on 16 CTAs, LiDAR chain of 20,876 points: 343 / 291 / 275 / 288 / 320 us)
@@ -479,7 +484,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
     SmallSmem& sm = smem();
     if (threadIdx.x == 0) {
         sm.nopen[0] = 0;
-        if (kRare) sm.ntwin = 0;
+        if (kRare && kW) sm.ntwin = 0;
     }
     // group(i0, all): the points i0, i0 + T, ... of which `all`, or those below n, are there.
     // A thread's loops run over whole groups, free of range checks, and one more
@@ -492,7 +497,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
 #pragma unroll 1
         for (; i0 < n; i0 += kIn * T) group(i0, std::false_type{});
     };
-    if (kRare && pg->far) {
+    if (kRare && (!kW || pg->far)) {
         far_cells<SM, T>(stg, n, pg, word, mult, t0);
     } else {
         const CellMap cell(pg->bg);
@@ -513,7 +518,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
 #pragma unroll
             for (int k = 0; k < kIn; ++k) {
                 const int i = i0 + k * T;
-                if (kRare) c[k] = min(c[k], kNoCell - 1u);  // (kWide: any number)
+                if (kRare && kW) c[k] = min(c[k], kNoCell - 1u);  // (kWide: any number)
                 if (__float_as_int(q[k].w) < 0) c[k] = kNoCell;  // taken
                 if (all.value || i < n) {
                     area[i] = c[k];
@@ -552,14 +557,14 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
             if (c[k] != kNoCell) {
                 won += (w[k] == static_cast<unsigned>(i0 + k * T)) ? 1u : 0u;
                 bits |= (other != c[k]) ? (1u << k) : 0u;
-                if (kRare) eq |= (other == c[k] && w[k] != static_cast<unsigned>(i0 + k * T)) ? (1u << k) : 0u;
+                if (kRare && kW) eq |= (other == c[k] && w[k] != static_cast<unsigned>(i0 + k * T)) ? (1u << k) : 0u;
             }
         }
         left |= static_cast<unsigned long long>(bits) << k0;
-        if (kRare) same |= static_cast<unsigned long long>(eq) << k0;
+        if (kRare && kW) same |= static_cast<unsigned long long>(eq) << k0;
         k0 += kIn;
     });
-    const bool wide = kRare && pg->mode == kWide;
+    const bool wide = kRare && kW && pg->mode == kWide;
     if (wide) wide_check<SM>(stg, pg, word, nslots, mult, same, t0, T, nullptr);
     unsigned short* const list = reinterpret_cast<unsigned short*>(dyn + kListOff);
     append_open(left, t0, T, list, kOpenA);
@@ -567,7 +572,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
     int c = sm.nopen[0];
     unsigned more;
     if (c <= kOpenA) {
-        more = settle_open<SM, kRare>(stg, pg, word, nslots, c, list, kOpenA, list + kOpenA, kSelMax - kOpenA);
+        more = settle_open<SM, kRare && kW>(stg, pg, word, nslots, c, list, kOpenA, list + kOpenA, kSelMax - kOpenA);
     } else {
         // too many for the list (levels near 32,768 points in about as many cells):
         // half of the words, which are done with, take it
@@ -579,7 +584,7 @@ __device__ __noinline__ unsigned count_cells(const float4* stg, int n, const Pas
         __syncthreads();
         c = sm.nopen[0];
         if (c > half) return kManyOpen;
-        more = settle_open<SM, kRare>(stg, pg, word, half, c, word + half, half, list, kSelMax);
+        more = settle_open<SM, kRare && kW>(stg, pg, word, half, c, word + half, half, list, kSelMax);
     }
     if (more == kManyOpen) return kManyOpen;
     won += more;
@@ -685,27 +690,30 @@ __device__ __noinline__ unsigned count_index(const float4* src, int n, const Pas
     return fresh;
 }
 
-// The voxels of a size that this thread's points (t0, t0 + T, ...) count.  (On one CTA,
-// whose few points hardly repay the code, far boxes and kWide take the general
-// ways: with them 1,000 points took 48.3 us, without 47.2.)
-template <bool SM, int T>
+// The voxels of a size that this thread's points (t0, t0 + T, ...) count.  (On one CTA
+// far boxes take the general way: its few points hardly repay the code, 1,000 points
+// 48.3 us with it, 47.2 without.)
+template <bool SM, int T, bool kW>
 __device__ __forceinline__ unsigned count_pass(const float4* stg, int n, const PassGrid* pg, int t0) {
     constexpr bool kCluster = T == kST;
     const int mode = pg->mode;
-    if (mode == kSkip) return 0u;
-    if (mode < kWide || (kCluster && mode == kWide)) {
-        const unsigned won = (kCluster && (mode == kWide || pg->far)) ? count_cells<SM, kST, true>(stg, n, pg, t0)
-                                                                      : count_cells<SM, T, false>(stg, n, pg, t0);
+    if (mode == kDirect || mode == kHash || (kW && mode == kWide)) {
+        const unsigned won = (kCluster && (pg->far || (kW && mode == kWide)))
+                                 ? count_cells<SM, kST, true, kW>(stg, n, pg, t0)
+                                 : count_cells<SM, T, false, kW>(stg, n, pg, t0);
         if (won != kManyOpen) return won;
-        if (mode != kWide) return count_open<SM, T>(n, pg, t0);
+        if (!kW || mode != kWide) return count_open<SM, T>(n, pg, t0);
         __syncthreads();  // (the count's area is filled anew)
+        return count_index<SM, T>(stg, n, pg, t0);
     }
-    return count_index<SM, T>(stg, n, pg, t0);
+    if (mode == kIndex) return count_index<SM, T>(stg, n, pg, t0);
+    return 0u;
 }
 
 // The grids of up to ten sizes over the level's box into sm.pg[first ...], how
 // a pass counts them, by one warp: lanes [3 o, 3 o + 3) take size o (sv, alike
 // in those lanes), a lane per axis.
+template <bool kW>
 __device__ __noinline__ void set_grids(int first, int sizes, float sv, const float* aspect, int n, unsigned area_words) {
     SmallSmem& sm = smem();
     const int lane = threadIdx.x & 31;
@@ -735,7 +743,7 @@ __device__ __noinline__ void set_grids(int first, int sizes, float sv, const flo
             const unsigned words = 2u * (area_words - static_cast<unsigned>(n));
             const bool direct = fast && cells <= words;
             g.sv = sv;
-            g.mode = !fast ? (all_ok ? kIndex : kSkip) : (direct ? kDirect : (cells < kNoCell ? kHash : kWide));
+            g.mode = !fast ? (all_ok ? kIndex : kSkip) : (direct ? kDirect : (cells < kNoCell ? kHash : (kW ? kWide : kIndex)));
             g.nslots = direct ? static_cast<unsigned>(cells) : min(words, 4u * static_cast<unsigned>(n));
             g.far = isinf(vmax) ? 1 : 0;
             g.bg.amb = __fmul_rn(vmax, kNear);
@@ -816,7 +824,7 @@ __device__ __forceinline__ void select_insert(SmallSmem& sm, bool in, unsigned l
 
 // Levels [first_level, P.L) of every segment; level first_level > 0 reads its
 // input through orig[(first_level - 1) & 1].
-template <int Q>
+template <int Q, bool kW>
 __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
     hav_small_kernel(const __grid_constant__ Plan P, int first_level) {
     cg::cluster_group cl = cg::this_cluster();
@@ -1051,17 +1059,17 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                     int t = sm.t, par = 0, cur = 0;
                     if (t < steps) {
                         if (wid == kWarps - 1)
-                            set_grids(0, 1, next_size(lo, hi, up, sm.first), P.aspect, n, area_words);
+                            set_grids<kW>(0, 1, next_size(lo, hi, up, sm.first), P.aspect, n, area_words);
                         __syncthreads();
                         for (;;) {
                             const PassGrid& pg = sm.pg[cur];
                             const float sv = pg.sv;
                             const bool fits = pg.bg.ok != 0;  // (alike in every thread)
                             if (wid == kWarps - 1)  // outcome 0: too many voxels, 1: too few
-                                set_grids(2 * (par ^ 1), 2,
+                                set_grids<kW>(2 * (par ^ 1), 2,
                                           lane < 3 ? next_size(sv, hi, up, 0.0f) : next_size(lo, sv, false, 0.0f),
                                           P.aspect, n, area_words);
-                            const unsigned won = __reduce_add_sync(0xffffffffu, count_pass<true, T>(pts, n, &pg, t0));
+                            const unsigned won = __reduce_add_sync(0xffffffffu, count_pass<true, T, false>(pts, n, &pg, t0));
                             if (lane == 0) sm.wcnt[par][wid] = won;
                             __syncthreads();
                             const int K = static_cast<int>(
@@ -1101,7 +1109,7 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                     if (tid == 0) sm.t = t;
                     if (!accepted) {
                         s_star = fixed ? P.fixed_s : (P.t_max == 0 ? sm.s_hi : (lo > 0.0f ? lo : hi));
-                        if (wid == 0) set_grids(4, 1, s_star, P.aspect, n, area_words);
+                        if (wid == 0) set_grids<kW>(4, 1, s_star, P.aspect, n, area_words);
                         __syncthreads();
                     }
                 } else {
@@ -1186,7 +1194,7 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                             const float ns = cand_size(lo, hi, up, first, lane < kNodes ? lane : 0);
                             if (lane < kNodes) sm.node_s[lane] = ns;
                             const float sv = __shfl_sync(0xffffffffu, ns, (lane < 3 && rank < kNodes) ? rank : 0);
-                            set_grids(go ? 0 : 4, go ? 2 : 1, go ? sv : ss, P.aspect, n, area_words);
+                            set_grids<kW>(go ? 0 : 4, go ? 2 : 1, go ? sv : ss, P.aspect, n, area_words);
                             if (lane == 0 && go) {
                                 // left out: a step beyond the last, and a slower way to count
                                 // than the root's (much finer sizes: the search seldom gets there)
@@ -1199,8 +1207,8 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
                         }
                         __syncthreads();
                         if (!sm.go) break;
-                        unsigned won = in_smem ? count_pass<true, kST>(pts, n, sm.pg, tid)
-                                               : count_pass<false, kST>(stg, n, sm.pg, tid);
+                        unsigned won = in_smem ? count_pass<true, kST, kW>(pts, n, sm.pg, tid)
+                                               : count_pass<false, kST, kW>(stg, n, sm.pg, tid);
                         won = __reduce_add_sync(0xffffffffu, won);
                         if (lane == 0) sm.wcnt[0][wid] = won;
                         __syncthreads();
@@ -1545,46 +1553,46 @@ __global__ void __cluster_dims__(Q, 1, 1) __launch_bounds__(kST, 1)
 
 }  // namespace
 
+// Sets a cluster kernel's launch attributes; the clusters that run at once, or -1.
+template <int Q, bool kW>
+static int set_up(cudaLaunchConfig_t* cfg) {
+    int nc = 0;
+    if (cudaFuncSetAttribute(hav_small_kernel<Q, kW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kSmallDyn)) != cudaSuccess)
+        return -1;
+    if (Q == 1) return 1;
+    if (Q > 8 && cudaFuncSetAttribute(hav_small_kernel<Q, kW>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                     cudaSuccess)
+        return -1;
+    return cudaOccupancyMaxActiveClusters(&nc, hav_small_kernel<Q, kW>, cfg) == cudaSuccess ? nc : -1;
+}
+
 int small_clusters(int device, int q) {
     (void)device;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(q * 16));
     cfg.blockDim = dim3(kST);
     cfg.dynamicSmemBytes = kSmallDyn;
-    int nc = 0;
-    if (q == 1) {
-        if (cudaFuncSetAttribute(hav_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kSmallDyn)) != cudaSuccess)
-            return -1;
-        return 1;
-    }
-    if (q == 8) {
-        if (cudaFuncSetAttribute(hav_small_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kSmallDyn)) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&nc, hav_small_kernel<8>, &cfg) != cudaSuccess)
-            return -1;
-        return nc;
-    }
-    if (q == 16) {
-        if (cudaFuncSetAttribute(hav_small_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kSmallDyn)) != cudaSuccess ||
-            cudaFuncSetAttribute(hav_small_kernel<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&nc, hav_small_kernel<16>, &cfg) != cudaSuccess)
-            return -1;
-        return nc;
-    }
-    return -1;
+    if (q == 1) return set_up<1, false>(&cfg);
+    if (q != 8 && q != 16) return -1;
+    const int a = q == 8 ? set_up<8, false>(&cfg) : set_up<16, false>(&cfg);
+    const int b = q == 8 ? set_up<8, true>(&cfg) : set_up<16, true>(&cfg);
+    return a < b ? a : b;
 }
 
 int launch_small(const Plan& plan, int first_level, int q, int nclusters, cudaStream_t stream) {
     if (q != 8 && q != 16) return -1;
-    // every level of the launch must fit its cluster's shared memory
+    // every level of the launch must fit its cluster's shared memory; sizes of 2^32
+    // cells and more (kWide) are seldom met but near the points' own spacing, with
+    // budgets of nearly all points (LiDAR scans of 16,384 points to 97 of 100 155 us
+    // by kIndex, 94 by kWide; to 9/10 equal, of 24,000 151 and 97)
+    bool wide = false;
     for (int j = first_level; j < plan.L; ++j)
 #pragma unroll 1
         for (int s = 0; s < plan.S; ++s) {
             const long long n = (j == 0) ? plan.off0[s + 1] - plan.off0[s] : plan.m[j - 1][s];
             if (n > static_cast<long long>(kSmallMax)) return -1;
+            wide = wide || (n > kWideMin && 8ll * plan.m[j][s] >= 7 * n);
         }
     int nc = nclusters < plan.S ? nclusters : plan.S;
     if (nc < 1) nc = 1;
@@ -1593,8 +1601,11 @@ int launch_small(const Plan& plan, int first_level, int q, int nclusters, cudaSt
     cfg.blockDim = dim3(kST);
     cfg.dynamicSmemBytes = kSmallDyn;
     cfg.stream = stream;
-    const cudaError_t e = (q == 16) ? cudaLaunchKernelEx(&cfg, hav_small_kernel<16>, plan, first_level)
-                                    : cudaLaunchKernelEx(&cfg, hav_small_kernel<8>, plan, first_level);
+    const cudaError_t e =
+        wide ? (q == 16 ? cudaLaunchKernelEx(&cfg, hav_small_kernel<16, true>, plan, first_level)
+                        : cudaLaunchKernelEx(&cfg, hav_small_kernel<8, true>, plan, first_level))
+             : (q == 16 ? cudaLaunchKernelEx(&cfg, hav_small_kernel<16, false>, plan, first_level)
+                        : cudaLaunchKernelEx(&cfg, hav_small_kernel<8, false>, plan, first_level));
     return e == cudaSuccess ? 1 : -1;
 }
 
@@ -1612,7 +1623,7 @@ int launch_solo(const Plan& plan, int first_level, int nblocks, cudaStream_t str
     cfg.blockDim = dim3(kST);
     cfg.dynamicSmemBytes = kSmallDyn;
     cfg.stream = stream;
-    return cudaLaunchKernelEx(&cfg, hav_small_kernel<1>, plan, first_level) == cudaSuccess ? 1 : -1;
+    return cudaLaunchKernelEx(&cfg, hav_small_kernel<1, false>, plan, first_level) == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace havk

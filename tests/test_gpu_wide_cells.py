@@ -119,7 +119,7 @@ def twins(pairs, repeats, seed):
 
 
 # cells whose numbers agree modulo 2^32: few, and more than are collected
-@pytest.mark.parametrize("pairs,repeats", [(3, 3), (200, 2), (900, 2), (1900, 1), (5000, 2), (15000, 1)])
+@pytest.mark.parametrize("pairs,repeats", [(3, 3), (900, 2), (1900, 1), (200, 30), (900, 8), (5000, 2), (15000, 1)])
 def test_twins(hv, ctx, pairs, repeats):
     pts = twins(pairs, repeats, pairs)
     tro = check(hv, ctx, pts, [len(pts)], layers=1)  # (never enough voxels: every size of the search)
