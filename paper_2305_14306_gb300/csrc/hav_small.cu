@@ -1584,8 +1584,8 @@ int launch_small(const Plan& plan, int first_level, int q, int nclusters, cudaSt
     if (q != 8 && q != 16) return -1;
     // every level of the launch must fit its cluster's shared memory; sizes of 2^32
     // cells and more (kWide) are seldom met but near the points' own spacing, with
-    // budgets of nearly all points (LiDAR scans of 16,384 points to 97 of 100 155 us
-    // by kIndex, 94 by kWide; to 9/10 equal, of 24,000 151 and 97)
+    // budgets of nearly all points (LiDAR scans of 16,384 points to 97 of 100 156 us
+    // by kIndex, 91 by kWide; to 9/10 equal, of 24,000 151 and 97)
     bool wide = false;
     for (int j = first_level; j < plan.L; ++j)
 #pragma unroll 1
